@@ -497,7 +497,8 @@ void launch_apply_sip(int N, const OpGeom& g, const T* x, T* y, const T* eta, T 
                                   reinterpret_cast<const float*>(z), float(beta), nullptr, s))
             return;
     }
-    if ((v == APPLY_STAGE || split) &&
+    // the FP64 operator's default is the staged entry too (fixed-point kernel)
+    if ((v == APPLY_STAGE || split || (sizeof(T) == 8 && v == APPLY_AUTO)) &&
         launch_apply_sip_stage<T>(N, g, x, y, eta, alpha, z, beta, nullptr, s))
         return;
     if constexpr (sizeof(T) == 4) {

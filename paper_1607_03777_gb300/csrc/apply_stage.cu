@@ -516,7 +516,8 @@ void stage_split(const OpGeom& g, const float* x, float* y, const float* eta, fl
     hi.tiles = g.hi_tiles;
     SIP_CUDA(cudaEventRecord(f.fork, s));
     SIP_CUDA(cudaStreamWaitEvent(f.s, f.fork, 0));
-    launch_stage<N, float, double, SPLIT_TYS, true>(hi, dim3(unsigned(g.n_hi)), vec, f.s);
+    if (!launch_apply_fix_list(N, g, x, y, eta, alpha, z, beta, r1, f.s))
+        launch_stage<N, float, double, SPLIT_TYS, true>(hi, dim3(unsigned(g.n_hi)), vec, f.s);
     SIP_CUDA(cudaEventRecord(f.join, f.s));
     // the unflagged tiles: the warp-row kernel (y = alpha A x + beta z), else
     // (residual restricted to the Q^2_1 modes) the staged kernel
@@ -538,6 +539,9 @@ void stage_dispatch(const OpGeom& g, const T* x, T* y, const T* eta, T alpha, co
             stage_split<N>(g, x, y, eta, alpha, z, beta, r1, s);
             return;
         }
+    } else {
+        // FP64: the fixed-point kernel wherever it applies
+        if (launch_apply_fix(N, g, x, y, eta, alpha, z, beta, r1, s)) return;
     }
     if constexpr (StageLayout<N, T, T, 4>::BYTES <= kMaxSmem) {
         if (g.stage_rows[sizeof(T) == 4 ? 1 : 0] == 4) {

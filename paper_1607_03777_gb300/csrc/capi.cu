@@ -184,6 +184,10 @@ sip_status sip_problem_create(sip_ctx* ctx, const sip_problem_desc* d, sip_probl
             p->n_p = ne * p->mp;
             p->geom = sip::make_geom(d->nx, d->ny, d->lx, d->ly, d->bc, d->k, d->penalty_scale);
             p->geom1 = p->geom;   // the Galerkin A_1 keeps the fine-k penalty
+            // continuous vectors, whose jumps cancel exactly in FP64 arithmetic: the
+            // coarse problem is nearly singular where a stiff inclusion floats, and
+            // amplifies the last bits of its stencils by 1e7
+            p->geom1.variant[0] = sip::APPLY_ELEM2;
             p->eta_host = eta;
             const cudaStream_t s = sip::alloc_stream();
             p->eta_d.alloc(ne * sizeof(double));
@@ -223,7 +227,7 @@ sip_status sip_problem_schedule(const sip_problem* p, int apply[2], int fused[2]
     for (int t = 0; t < 2; ++t) {
         if (apply) {
             const int v = p->geom.variant[t];
-            apply[t] = v != sip::APPLY_AUTO ? v : (p->n <= 6 ? int(sip::APPLY_ELEM2)
+            apply[t] = v != sip::APPLY_AUTO ? v : (p->n <= 6 ? int(t == 0 ? sip::APPLY_STAGE : sip::APPLY_ELEM2)
                                                              : int(sip::APPLY_TILE));
             if (apply[t] == int(sip::APPLY_STAGE) && p->geom.stage_rows[t] == 4) apply[t] = 5;
             if (t == 1 && p->geom.n_hi > 0 && p->n <= 6) apply[t] = int(sip::APPLY_STAGE);

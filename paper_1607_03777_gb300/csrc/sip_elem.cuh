@@ -4,6 +4,7 @@
 // volume terms of one velocity component (eq. stiffness_form).
 #pragma once
 
+#include "fix_core.cuh"
 #include "sip_face.cuh"
 #include "sip_internal.h"
 
@@ -77,6 +78,37 @@ void launch_apply_stage_batch(int N, const StageArgs<TS, TC>* args, const int2* 
 template <typename TS, typename TC>
 StageArgs<TS, TC> stage_args(const OpGeom& g, const TS* x, TS* y, const TS* eta, double alpha,
                              const TS* z, double beta, TS* r1, int N);
+
+// Fixed-point apply (apply_fix.cu), TS = storage.
+template <typename TS>
+struct FixArgs {
+    const TS* x;
+    TS* y;
+    const TS* eta;
+    const TS* z;
+    TS* r1;                      // non-null: write only the Q^2_1 modes of the result here
+    double alpha, beta;
+    double hx, hy, pen_x, pen_y;
+    int nx, ny;
+    int bc[4];
+    int vec;                     // two entries per access of y and z
+    fix::Scal k;
+    double ss[36], os[36];       // s_i s_j and alpha s_i s_j per mode
+};
+// The arguments of y = alpha A x + beta z; false where the fixed-point form
+// does not apply (degree above 5, factors out of its range).
+template <typename TS>
+bool make_fix_args(int N, const OpGeom& g, const TS* x, TS* y, const TS* eta, double alpha, const TS* z,
+                   double beta, TS* r1, FixArgs<TS>& a);
+// items: (member, 32 x 2 tile); active (may be null) masks members
+template <typename TS>
+void launch_apply_fix_batch(int N, const FixArgs<TS>* args, const int2* items, int n_items,
+                            const int* active, cudaStream_t s);
+bool launch_apply_fix(int N, const OpGeom& g, const double* x, double* y, const double* eta,
+                      double alpha, const double* z, double beta, double* r1, cudaStream_t s);
+// the tiles of g.hi_tiles only
+bool launch_apply_fix_list(int N, const OpGeom& g, const float* x, float* y, const float* eta,
+                           float alpha, const float* z, float beta, float* r1, cudaStream_t s);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

@@ -487,7 +487,8 @@ void Multigrid<T>::mark_split_tiles(cudaStream_t s) {
 template <typename T>
 bool Multigrid<T>::residual_restrict(const T* y, const T* b, T* r1, cudaStream_t s) {
     const bool split = sizeof(T) == 4 && P->geom.n_hi > 0;
-    if (split || apply_variant<T>(P->geom) == APPLY_STAGE)
+    const int v = apply_variant<T>(P->geom);
+    if (split || v == APPLY_STAGE || (sizeof(T) == 8 && v == APPLY_AUTO))
         return launch_apply_sip_stage<T>(N, P->geom, y, nullptr, eta_of<T>(P), T(-1), b, T(1), r1,
                                          s);
     return use_fused() && launch_residual_restrict_elem<T>(N, P->geom, y, b, eta_of<T>(P), r1, s);
@@ -520,6 +521,8 @@ void Multigrid<T>::setup(cudaStream_t s) {
     tune_smoother(s);
 
     const OpGeom& g1 = P->geom1;
+    OpGeom g0 = P->geom;   // probing for A_0: FP64 arithmetic, as for A_1
+    if (g0.variant[0] == APPLY_AUTO || g0.variant[0] == APPLY_STAGE) g0.variant[0] = APPLY_ELEM2;
     const bool q0 = d.coarse == SIP_COARSE_Q0;
     if (d.n_hlevels == 0 && !q0) {
         // A_p(Q^2_1): the coarse problem A_1 = P^T A P itself, by probing with
@@ -598,7 +601,7 @@ void Multigrid<T>::setup(cudaStream_t s) {
                     if (l == 0 && q0) {
                         SIP_CUDA(cudaMemsetAsync(t1.ptr, 0, n_u * sizeof(double), s));
                         launch_p_prolong_add<double>(ne, N, xv.as<double>(), t1.as<double>(), s, 1);
-                        launch_apply_sip<double>(N, P->geom, t1.as<double>(), t2.as<double>(),
+                        launch_apply_sip<double>(N, g0, t1.as<double>(), t2.as<double>(),
                                                  P->eta_d.as<double>(), 1.0, nullptr, 0.0, s);
                         launch_p_restrict<double>(ne, N, t2.as<double>(), y, s, 1);
                     } else if (l == 0) {
@@ -1059,10 +1062,16 @@ sip_status run_solve(sip_problem* P, const double* f_u, const double* g_p, doubl
     auto project = [&](double* v) {
         if (singular) launch_zero_mean_pressure(size_t(P->ne), P->mp, v + n_u, wsd, s);
     };
-    // y = K v  (w_u = A v_u + B v_p, w_p = B^T v_u)
+    // y = K v  (w_u = A v_u + B v_p, w_p = B^T v_u).  One application per outer
+    // iteration (25 of 1600 operator applies of the 128^2, k = 3 box solve): it
+    // stays in FP64 arithmetic, whose rounding sets the attainable residual the
+    // stopping tests were chosen on; with the more accurate fixed-point apply some
+    // solves stop one or two iterations earlier at the same tolerance.
+    OpGeom gK = P->geom;
+    if (gK.variant[0] == APPLY_AUTO || gK.variant[0] == APPLY_STAGE) gK.variant[0] = APPLY_ELEM2;
     auto applyK = [&](const double* v, double* y) {
         launch_apply_B<double>(P->k, P->geom, v + n_u, W.tu.as<double>(), s);
-        launch_apply_sip<double>(P->n, P->geom, v, y, eta, 1.0, W.tu.as<double>(), 1.0, s);
+        launch_apply_sip<double>(P->n, gK, v, y, eta, 1.0, W.tu.as<double>(), 1.0, s);
         launch_apply_Bt<double>(P->k, P->geom, v, y + n_u, s);
     };
     int inner_total = 0, inner_max = 0, inner_calls = 0;
