@@ -301,6 +301,7 @@ struct BArgs {
     Tab1D<N, T> tab;
 };
 
+// Double-double instances (FP64: apply_div.cu).
 // B p: one thread per velocity output (e, c, jq, iq); N = k + 1, pressure
 // degree k - 1 (indices < K = N - 1).
 template <int N, typename T>
@@ -549,7 +550,6 @@ void launch_apply_B(int k, const OpGeom& g, const T* p, T* y, cudaStream_t s) {
     }
     SIP_CHECK_LAUNCH();
 }
-template void launch_apply_B<double>(int, const OpGeom&, const double*, double*, cudaStream_t);
 
 template <typename T>
 void launch_apply_Bt(int k, const OpGeom& g, const T* u, T* y, cudaStream_t s) {
@@ -564,7 +564,6 @@ void launch_apply_Bt(int k, const OpGeom& g, const T* u, T* y, cudaStream_t s) {
     }
     SIP_CHECK_LAUNCH();
 }
-template void launch_apply_Bt<double>(int, const OpGeom&, const double*, double*, cudaStream_t);
 
 // Double-double instances (residual of iterative refinement): the tile
 // kernel, B and B^T evaluate the same operator with the same FP64

@@ -257,7 +257,8 @@ constexpr int min_blocks() {
 template <int N, int TW, int TH, typename TS>
 __global__ void __launch_bounds__(TW* TH* N, (min_blocks<N, TW, TH>())) k_apply_fix(const FixArgs<TS> a) {
     grid_dep_wait();
-    fix_body<N, TW, TH, TS>(a, blockIdx.x * TW, blockIdx.y * TH);
+    const int ntx = (a.nx + TW - 1) / TW;   // 1D grid: no limit on mesh rows
+    fix_body<N, TW, TH, TS>(a, int(blockIdx.x % ntx) * TW, int(blockIdx.x / ntx) * TH);
 }
 
 // Tiles of 32 x 2 elements named by a list (split precision), two CTAs each.
@@ -297,7 +298,7 @@ void launch_tiles(const FixArgs<TS>& a, cudaStream_t s) {
         return true;
     }();
     (void)attr;
-    launch_k(k_apply_fix<N, TW, TH, TS>, dim3((a.nx + TW - 1) / TW, (a.ny + TH - 1) / TH),
+    launch_k(k_apply_fix<N, TW, TH, TS>, dim3(unsigned(((a.nx + TW - 1) / TW) * ((a.ny + TH - 1) / TH))),
              TW * TH * N, smem, s, a);
     SIP_CHECK_LAUNCH();
 }

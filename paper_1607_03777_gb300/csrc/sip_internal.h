@@ -248,6 +248,11 @@ template <typename T>
 void launch_apply_B(int k, const OpGeom& g, const T* p, T* y, cudaStream_t s);
 template <typename T>
 void launch_apply_Bt(int k, const OpGeom& g, const T* u, T* y, cudaStream_t s);
+// FP64: apply_div.cu; double-double: apply.cu
+template <>
+void launch_apply_B<double>(int k, const OpGeom& g, const double* p, double* y, cudaStream_t s);
+template <>
+void launch_apply_Bt<double>(int k, const OpGeom& g, const double* u, double* y, cudaStream_t s);
 void launch_rhs_body_force(int k, const OpGeom& g, const double* rho, double grav, double* f,
                            cudaStream_t s);
 void launch_rasterise(int nx, int ny, double lx, double ly, const double* shapes, int ns,
