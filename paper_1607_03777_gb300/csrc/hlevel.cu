@@ -1,0 +1,260 @@
+// One continuous level of the h-hierarchy in two launches: everything before
+// the coarse correction (Chebyshev / point-Jacobi steps from zero, residual,
+// restriction) and everything after it (interpolation, steps).
+//
+// What bounds it: latency.  A stencil application on a 129^2-vertex level is
+// 1 us of FP64 work and 4 MB from L2, but one launch per step takes about 4 us
+// in a replayed graph, nine per level.  Here a CTA runs all steps of its tile on
+// a halo that shrinks by one ring per application, one thread per (vertex,
+// component) with its stencil row in registers (read once instead of once per
+// step) and the direction in shared memory.  The rings are recomputed by the
+// neighbouring tiles: 2.0x the FP64 work at 12 x 12 vertices and three steps,
+// which is what limits the tile from below; large FP64 levels, where that work
+// outweighs the launches, keep one launch per step (fused_level_ok).
+#include "sip_internal.h"
+#include "sip_level.cuh"
+#include "sip_solver.h"
+
+namespace sip {
+
+namespace {
+
+constexpr int kMaxThreads = 768;
+constexpr int kMaxSteps = 4;
+
+template <typename T>
+struct HLevelArgs {
+    int nvx, nvy;     // vertices of this level
+    int ncx, ncy;     // intervals of the next one
+    const T* S;
+    const T* dinv;
+    const T* b;
+    const T* xin;     // after: the iterate before the correction
+    T* x;
+    const T* xc;      // after: coarse correction
+    T* bc;            // before: coarse right-hand side
+    T c1[kMaxSteps], c2[kMaxSteps];
+    int steps, tile, rw;   // coarse vertices of a tile, vertices of its region, per direction
+};
+
+template <typename T>
+__device__ __forceinline__ T row_dot(const T (&s)[18], const T* v, int rw) {
+    T acc = T(0);
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+            const T* w = v + 2 * ((dy - 1) * rw + dx - 1);
+            const int t = 2 * (dy * 3 + dx);
+            acc += s[t] * w[0] + s[t + 1] * w[1];
+        }
+    return acc;
+}
+
+template <typename T>
+__device__ __forceinline__ void load_row(const T* S, size_t g, T (&s)[18]) {
+    const T* p = S + (g / 2) * 36 + (g % 2) * 2;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) ld2<T, true>(p + 4 * t, s[2 * t], s[2 * t + 1]);
+}
+
+// One thread's place in its tile's region.
+struct Place {
+    bool in;       // inside the grid
+    int ring;      // distance from the region's edge
+    int node;      // 2 * (local vertex) + component
+    size_t g;      // global row
+    int gx, gy, c;
+};
+
+template <typename T>
+__device__ __forceinline__ Place place(const HLevelArgs<T>& a, int ox, int oy) {
+    Place p;
+    p.c = threadIdx.x % 2;
+    const int v = threadIdx.x / 2, lx = v % a.rw, ly = v / a.rw;
+    p.node = threadIdx.x;
+    p.gx = ox + lx;
+    p.gy = oy + ly;
+    p.in = ly < a.rw && p.gx >= 0 && p.gx < a.nvx && p.gy >= 0 && p.gy < a.nvy;
+    p.ring = min(min(lx, a.rw - 1 - lx), min(ly, a.rw - 1 - ly));
+    p.g = p.in ? 2 * (size_t(p.gy) * a.nvx + p.gx) + p.c : 0;
+    return p;
+}
+
+// x = Chebyshev steps on S x = b from zero; bc = R_h (b - S x).
+template <typename T>
+__global__ void __launch_bounds__(kMaxThreads) k_level_before(const HLevelArgs<T> a) {
+    grid_dep_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int nt = 2 * a.rw * a.rw;
+    T* sd = reinterpret_cast<T*>(smem_raw);   // direction, then iterate
+    T* sr = sd + nt;                          // residual
+    const int ntx = (a.ncx + a.tile) / a.tile;   // ceil((ncx + 1) / tile)
+    const int I0 = int(blockIdx.x % ntx) * a.tile, J0 = int(blockIdx.x / ntx) * a.tile;
+    const Place p = place(a, 2 * I0 - 1 - a.steps, 2 * J0 - 1 - a.steps);
+    const bool mine = int(threadIdx.x) < nt;
+    T s[18], r = T(0), d = T(0), x = T(0), bv = T(0), di = T(0);
+    if (p.in) {
+        bv = a.b[p.g];
+        di = a.dinv[p.g];
+        if (p.ring > 0) load_row(a.S, p.g, s);
+        r = bv;
+        x = d = a.c2[0] * di * bv;
+    }
+    if (mine) sd[p.node] = d;
+    __syncthreads();
+    for (int st = 1; st < a.steps; ++st) {
+        if (p.in && p.ring >= st) {
+            r -= row_dot(s, sd + p.node - p.c, a.rw);
+            d = a.c1[st] * d + a.c2[st] * di * r;
+            x += d;
+        }
+        __syncthreads();
+        if (mine) sd[p.node] = st + 1 < a.steps ? d : x;
+        __syncthreads();
+    }
+    if (mine) sr[p.node] = p.in && p.ring >= a.steps ? bv - row_dot(s, sd + p.node - p.c, a.rw) : T(0);
+    const int fx = p.gx - 2 * I0, fy = p.gy - 2 * J0, tf = 2 * a.tile;
+    if (p.in && fx >= 0 && fx < tf && fy >= 0 && fy < tf) a.x[p.g] = x;
+    __syncthreads();
+    for (int q = threadIdx.x; q < 2 * a.tile * a.tile; q += blockDim.x) {
+        const int c = q % 2, v = q / 2, I = I0 + v % a.tile, J = J0 + v / a.tile;
+        if (I > a.ncx || J > a.ncy) continue;
+        // the vertex in the region: 2 (I - I0) + 1 + steps
+        const T* w = sr + 2 * ((2 * (J - J0) + 1 + a.steps) * a.rw + 2 * (I - I0) + 1 + a.steps) + c;
+        T acc = T(0);
+        for (int dy = -1; dy <= 1; ++dy)
+            for (int dx = -1; dx <= 1; ++dx) {
+                const T wt = (dy == 0 ? T(1) : T(0.5)) * (dx == 0 ? T(1) : T(0.5));
+                acc += wt * w[2 * (dy * a.rw + dx)];   // zero outside the grid
+            }
+        a.bc[2 * (size_t(J) * (a.ncx + 1) + I) + c] = acc;
+    }
+}
+
+// x = Chebyshev steps on S x = b from xin + P_h xc.
+template <typename T>
+__global__ void __launch_bounds__(kMaxThreads) k_level_after(const HLevelArgs<T> a) {
+    grid_dep_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int nt = 2 * a.rw * a.rw;
+    T* sd = reinterpret_cast<T*>(smem_raw);
+    const int tf = 2 * a.tile, ntx = (a.nvx + tf - 1) / tf;
+    const int X0 = int(blockIdx.x % ntx) * tf, Y0 = int(blockIdx.x / ntx) * tf;
+    const Place p = place(a, X0 - a.steps, Y0 - a.steps);
+    const bool mine = int(threadIdx.x) < nt;
+    T s[18], r = T(0), d = T(0), x = T(0), bv = T(0), di = T(0);
+    if (p.in) {
+        bv = a.b[p.g];
+        di = a.dinv[p.g];
+        if (p.ring > 0) load_row(a.S, p.g, s);
+        const T* q = a.xc + 2 * (size_t(p.gy / 2) * (a.ncx + 1) + p.gx / 2) + p.c;
+        const int ux = p.gx % 2 ? 2 : 0, uy = p.gy % 2 ? 2 * (a.ncx + 1) : 0;
+        T v = q[0];
+        if (ux && uy) v = T(0.25) * (q[0] + q[ux] + q[uy] + q[ux + uy]);
+        else if (ux || uy) v = T(0.5) * (q[0] + q[ux + uy]);
+        x = a.xin[p.g] + v;
+    }
+    if (mine) sd[p.node] = x;
+    __syncthreads();
+    if (p.in && p.ring >= 1) {
+        r = bv - row_dot(s, sd + p.node - p.c, a.rw);
+        d = a.c2[0] * di * r;
+    }
+    T pend = d;
+    for (int st = 1; st < a.steps; ++st) {
+        __syncthreads();
+        if (mine) sd[p.node] = d;
+        __syncthreads();
+        if (p.in && p.ring >= st + 1) {
+            r -= row_dot(s, sd + p.node - p.c, a.rw);
+            d = a.c1[st] * d + a.c2[st] * di * r;
+            x += pend + d;
+            pend = T(0);
+        }
+    }
+    if (a.steps == 1) x += d;
+    const int fx = p.gx - X0, fy = p.gy - Y0;
+    if (p.in && fx >= 0 && fx < tf && fy >= 0 && fy < tf) a.x[p.g] = x;
+}
+
+// Coarse vertices per tile and direction: the largest (least recomputation)
+// that still gives most SMs a tile.
+int level_tile(int nvxc, int nvyc, int steps) {
+    for (int t = 6; t > 2; --t) {
+        const int rw = 2 * t + 1 + 2 * steps;
+        if (2 * rw * rw > kMaxThreads) continue;
+        if (((nvxc + t - 1) / t) * ((nvyc + t - 1) / t) >= 110) return t;
+    }
+    return 2;
+}
+
+template <typename T>
+HLevelArgs<T> level_args(const HLevel<T>& L, const HLevel<T>& C, int steps, const T* c1, const T* c2) {
+    HLevelArgs<T> a{};
+    a.nvx = L.nvx;
+    a.nvy = L.nvy;
+    a.ncx = C.nx;
+    a.ncy = C.ny;
+    a.S = L.S.template as<T>();
+    a.dinv = L.dinv.template as<T>();
+    a.b = L.b.template as<T>();
+    a.steps = steps;
+    a.tile = level_tile(C.nvx, C.nvy, steps);
+    for (int i = 0; i < steps; ++i) {
+        a.c1[i] = c1[i];
+        a.c2[i] = c2[i];
+    }
+    return a;
+}
+
+inline unsigned round32(int n) { return unsigned((n + 31) / 32 * 32); }
+
+}  // namespace
+
+template <typename T>
+bool fused_level_ok(const HLevel<T>& L, int steps) {
+    if (steps < 1 || steps > kMaxSteps) return false;
+    const int rw = 2 * 2 + 1 + 2 * steps;
+    if (2 * rw * rw > kMaxThreads) return false;
+    return sizeof(T) == 4 || size_t(L.nvx) * L.nvy <= size_t(300) * 300;
+}
+template bool fused_level_ok<float>(const HLevel<float>&, int);
+template bool fused_level_ok<double>(const HLevel<double>&, int);
+
+template <typename T>
+void launch_level_before(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, T* x,
+                         cudaStream_t s) {
+    HLevelArgs<T> a = level_args(L, C, steps, c1, c2);
+    a.rw = 2 * a.tile + 1 + 2 * steps;
+    a.x = x;
+    a.bc = C.b.template as<T>();
+    const int nt = 2 * a.rw * a.rw, t = a.tile;
+    const unsigned grid = unsigned(((C.nvx + t - 1) / t) * ((C.nvy + t - 1) / t));
+    launch_k(k_level_before<T>, grid, round32(nt), size_t(2 * nt) * sizeof(T), s, a);
+    SIP_CHECK_LAUNCH();
+}
+template void launch_level_before<float>(HLevel<float>&, HLevel<float>&, int, const float*, const float*,
+                                         float*, cudaStream_t);
+template void launch_level_before<double>(HLevel<double>&, HLevel<double>&, int, const double*,
+                                          const double*, double*, cudaStream_t);
+
+template <typename T>
+void launch_level_after(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, const T* xin,
+                        T* x, cudaStream_t s) {
+    HLevelArgs<T> a = level_args(L, C, steps, c1, c2);
+    a.rw = 2 * a.tile + 2 * steps;
+    a.xin = xin;
+    a.x = x;
+    a.xc = C.x.template as<T>();
+    const int nt = 2 * a.rw * a.rw, tf = 2 * a.tile;
+    const unsigned grid = unsigned(((L.nvx + tf - 1) / tf) * ((L.nvy + tf - 1) / tf));
+    launch_k(k_level_after<T>, grid, round32(nt), size_t(nt) * sizeof(T), s, a);
+    SIP_CHECK_LAUNCH();
+}
+template void launch_level_after<float>(HLevel<float>&, HLevel<float>&, int, const float*, const float*,
+                                        const float*, float*, cudaStream_t);
+template void launch_level_after<double>(HLevel<double>&, HLevel<double>&, int, const double*,
+                                         const double*, const double*, double*, cudaStream_t);
+
+}  // namespace sip

@@ -53,6 +53,9 @@ void launch_p_restrict(size_t ne, int N, const T* r, T* r1, cudaStream_t s, int 
 template <typename T>
 void launch_p_prolong_add(size_t ne, int N, const T* e1, T* y, cudaStream_t s, int M = 2);
 template <typename T> void launch_pcd(int nx, int ny, const T* v, T* out, cudaStream_t s);
+// y += P P_cd v on the Q^2_1 modes of y (degree N - 1)
+template <typename T>
+void launch_pcd_add(int nx, int ny, int N, const T* v, T* y, cudaStream_t s);
 template <typename T> void launch_rdc(int nx, int ny, const T* r, T* out, cudaStream_t s);
 template <typename T>
 void launch_stencil_apply(int nvx, int nvy, const T* S, const T* x, T* y, T alpha, const T* z,
@@ -126,6 +129,17 @@ struct HLevel {
     DeviceBuffer S, dinv, b, x, r, d, d2;
     double lmax = 0.0;
 };
+
+// ---- hlevel.cu: a level's work before and after its coarse correction, one
+// launch each (Chebyshev coefficients c1, c2 per step; x, xin: iterate buffers
+// that differ).  fused_level_ok: number of steps and level size it serves.
+template <typename T> bool fused_level_ok(const HLevel<T>& L, int steps);
+template <typename T>
+void launch_level_before(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, T* x,
+                         cudaStream_t s);
+template <typename T>
+void launch_level_after(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, const T* xin,
+                        T* x, cudaStream_t s);
 
 template <typename T>
 struct Multigrid {

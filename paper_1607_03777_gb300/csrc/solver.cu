@@ -746,17 +746,16 @@ void Multigrid<T>::smooth_p(const T* b, T* y, bool zero, cudaStream_t s) {
         }
         return;
     }
-    if (zero)
-        launch_axpby<T>(n_u, T(1), b, T(0), r, s);
-    else
-        launch_apply_sip<T>(N, P->geom, y, r, eta, T(-1), b, T(1), s);   // r = b - A y
+    // from zero the first residual is b itself: read where it lies
+    if (!zero) launch_apply_sip<T>(N, P->geom, y, r, eta, T(-1), b, T(1), s);   // r = b - A y
+    const T* r0 = zero ? b : r;
     double rho = 1.0 / ch.sigma;
     const T* einv = eta_inv_of<T>(P);
-    launch_bj_apply<T>(N, int(ne), r, dd, y, emap.as<int>(), cls_inv.template as<T>(),
+    launch_bj_apply<T>(N, int(ne), r0, dd, y, emap.as<int>(), cls_inv.template as<T>(),
                        cls_sym.as<int>(), uniq_inv.template as<T>(), einv,
                        T(0), T(1.0 / ch.theta), zero, s, bj_hi(), bj_inv64());
     for (int st = 1; st < P->desc.cheb_steps_p; ++st) {
-        launch_apply_sip<T>(N, P->geom, dd, r, eta, T(-1), r, T(1), s);  // r -= A d
+        launch_apply_sip<T>(N, P->geom, dd, r, eta, T(-1), st == 1 ? r0 : r, T(1), s);  // r -= A d
         const double rn = 1.0 / (2.0 * ch.sigma - rho);
         launch_bj_apply<T>(N, int(ne), r, dd, y, emap.as<int>(), cls_inv.template as<T>(),
                            cls_sym.as<int>(), uniq_inv.template as<T>(),
@@ -808,10 +807,29 @@ void Multigrid<T>::hcycle(int l, cudaStream_t s) {
         launch_dense_symv<T>(nc, cinv.template as<T>(), Lv.b.template as<T>(), Lv.x.template as<T>(), s);
         return;
     }
+    HLevel<T>& C = h[l + 1];
+    const int steps = P->desc.cheb_steps_h;
+    if (fused_level_ok(Lv, steps)) {
+        const Cheb ch(P->desc.cheb_lo * Lv.lmax, P->desc.cheb_hi * Lv.lmax);
+        std::vector<T> c1(steps), c2(steps);
+        c1[0] = T(0);
+        c2[0] = T(1.0 / ch.theta);
+        double rho = 1.0 / ch.sigma;
+        for (int st = 1; st < steps; ++st) {
+            const double rn = 1.0 / (2.0 * ch.sigma - rho);
+            c1[st] = T(rn * rho);
+            c2[st] = T(2.0 * rn / ch.delta);
+            rho = rn;
+        }
+        T* x0 = Lv.d.template as<T>();
+        launch_level_before<T>(Lv, C, steps, c1.data(), c2.data(), x0, s);
+        hcycle(l + 1, s);
+        launch_level_after<T>(Lv, C, steps, c1.data(), c2.data(), x0, Lv.x.template as<T>(), s);
+        return;
+    }
     smooth_h(l, true, s);
     launch_stencil_apply<T>(Lv.nvx, Lv.nvy, Lv.S.template as<T>(), Lv.x.template as<T>(), Lv.r.template as<T>(), T(-1),
                             Lv.b.template as<T>(), T(1), s);
-    HLevel<T>& C = h[l + 1];
     launch_rh<T>(C.nx, C.ny, Lv.r.template as<T>(), C.b.template as<T>(), s);
     hcycle(l + 1, s);
     launch_ph_add<T>(C.nx, C.ny, C.x.template as<T>(), Lv.x.template as<T>(), s);
@@ -859,8 +877,14 @@ void Multigrid<T>::vcycle_on(const T* b, T* y, cudaStream_t s) {
         launch_apply_sip<T>(N, P->geom, y, pr.template as<T>(), eta_of<T>(P), T(-1), b, T(1), s);
         launch_p_restrict<T>(ne, N, pr.template as<T>(), r1.template as<T>(), s);
     }
-    coarse_solve(r1.template as<T>(), e1.template as<T>(), s);
-    launch_p_prolong_add<T>(ne, N, e1.template as<T>(), y, s);
+    if (h.empty()) {
+        coarse_solve(r1.template as<T>(), e1.template as<T>(), s);
+        launch_p_prolong_add<T>(ne, N, e1.template as<T>(), y, s);
+    } else {   // P P_cd in one launch
+        launch_rdc<T>(P->desc.nx, P->desc.ny, r1.template as<T>(), h[0].b.template as<T>(), s);
+        hcycle(0, s);
+        launch_pcd_add<T>(P->desc.nx, P->desc.ny, N, h[0].x.template as<T>(), y, s);
+    }
     smooth_p(b, y, false, s);
 }
 

@@ -57,6 +57,23 @@ __global__ void k_pcd(int nx, int ny, const T* __restrict__ v, T* __restrict__ o
     out[g] = T(acc);
 }
 
+// The same added to the Q^2_1 modes of a degree N - 1 vector.
+template <typename T>
+__global__ void k_pcd_add(int nx, int ny, int N, const T* __restrict__ v, T* __restrict__ y) {
+    grid_dep_wait();
+    const size_t g = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const size_t ne = size_t(nx) * ny;
+    if (g >= ne * 8) return;
+    const size_t e = g / 8;
+    const int l = int(g % 8), c = l / 4, j = (l / 2) % 2, i = l % 2;
+    const int ex = int(e % nx), ey = int(e / nx);
+    double acc = 0.0;
+    for (int q = 0; q < 2; ++q)
+        for (int p = 0; p < 2; ++p)
+            acc += hatw(i, p) * hatw(j, q) * double(v[2 * (size_t(ey + q) * (nx + 1) + ex + p) + c]);
+    y[e * 2 * N * N + c * N * N + j * N + i] += T(acc);
+}
+
 template <typename T>
 __global__ void k_rdc(int nx, int ny, const T* __restrict__ r, T* __restrict__ out) {
     grid_dep_wait();
@@ -341,6 +358,11 @@ void launch_pcd(int nx, int ny, const T* v, T* out, cudaStream_t s) {
     SIP_CHECK_LAUNCH();
 }
 template <typename T>
+void launch_pcd_add(int nx, int ny, int N, const T* v, T* y, cudaStream_t s) {
+    launch_k(k_pcd_add<T>, nblk(size_t(nx) * ny * 8), 256, 0, s, nx, ny, N, v, y);
+    SIP_CHECK_LAUNCH();
+}
+template <typename T>
 void launch_rdc(int nx, int ny, const T* r, T* out, cudaStream_t s) {
     launch_k(k_rdc<T>, nblk(size_t(nx + 1) * (ny + 1) * 2), 256, 0, s, nx, ny, r, out);
     SIP_CHECK_LAUNCH();
@@ -438,6 +460,7 @@ void launch_convert(size_t n, const double* a, T* b, cudaStream_t s) {
     template void launch_p_restrict<T>(size_t, int, const T*, T*, cudaStream_t, int);           \
     template void launch_p_prolong_add<T>(size_t, int, const T*, T*, cudaStream_t, int);        \
     template void launch_pcd<T>(int, int, const T*, T*, cudaStream_t);                          \
+    template void launch_pcd_add<T>(int, int, int, const T*, T*, cudaStream_t);                 \
     template void launch_rdc<T>(int, int, const T*, T*, cudaStream_t);                          \
     template void launch_stencil_apply<T>(int, int, const T*, const T*, T*, T, const T*, T,     \
                                           cudaStream_t);                                         \
