@@ -273,20 +273,26 @@ __global__ void __launch_bounds__(32 * N, (min_blocks<N, 16, 2>())) k_apply_fix_
     fix_body<N, 16, 2, TS>(a, ex0, (t / ntx) * 2);
 }
 
-// Many operators in one launch: CTAs 2b and 2b + 1 apply the operator of member
-// items[b].x on its 32 x 2 tile items[b].y; members with active[m] == 0 are skipped.
-template <int N, typename TS>
+// Many operators in one launch, members with active[m] == 0 skipped.  SPLIT: CTAs
+// 2b and 2b + 1 apply the operator of member items[b].x on its 32 x 2 tile
+// items[b].y (split-precision tiles); else CTA b on its 8 x 4 tile.
+template <int N, typename TS, bool SPLIT>
 __global__ void __launch_bounds__(32 * N, (min_blocks<N, 16, 2>()))
     k_apply_fix_batch(const FixArgs<TS>* __restrict__ args, const int2* __restrict__ items,
                       const int* __restrict__ active) {
     grid_dep_wait();
-    const int2 it = items[blockIdx.x >> 1];
+    const int2 it = items[SPLIT ? blockIdx.x >> 1 : blockIdx.x];
     if (active && !active[it.x]) return;
     const FixArgs<TS>& a = args[it.x];
-    const int ntx = (a.nx + 31) / 32;
-    const int ex0 = (it.y % ntx) * 32 + (blockIdx.x & 1) * 16;
-    if (ex0 >= a.nx) return;
-    fix_body<N, 16, 2, TS>(a, ex0, (it.y / ntx) * 2);
+    if constexpr (SPLIT) {
+        const int ntx = (a.nx + 31) / 32;
+        const int ex0 = (it.y % ntx) * 32 + (blockIdx.x & 1) * 16;
+        if (ex0 >= a.nx) return;
+        fix_body<N, 16, 2, TS>(a, ex0, (it.y / ntx) * 2);
+    } else {
+        const int ntx = (a.nx + 7) / 8;
+        fix_body<N, 8, 4, TS>(a, (it.y % ntx) * 8, (it.y / ntx) * 4);
+    }
 }
 
 template <int N, int TW, int TH, typename TS>
@@ -328,16 +334,17 @@ void launch_list(const FixArgs<float>& a, const int* tiles, int n, cudaStream_t 
     SIP_CHECK_LAUNCH();
 }
 
-template <int N, typename TS>
+template <int N, typename TS, bool SPLIT>
 void launch_batch(const FixArgs<TS>* args, const int2* items, int n, const int* active, cudaStream_t s) {
-    constexpr size_t smem = fix::Tile<N, 16, 2>::BYTES;
+    constexpr size_t smem = SPLIT ? fix::Tile<N, 16, 2>::BYTES : fix::Tile<N, 8, 4>::BYTES;
     static const bool attr = [] {
-        SIP_CUDA(cudaFuncSetAttribute(k_apply_fix_batch<N, TS>,
+        SIP_CUDA(cudaFuncSetAttribute(k_apply_fix_batch<N, TS, SPLIT>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
         return true;
     }();
     (void)attr;
-    launch_k(k_apply_fix_batch<N, TS>, dim3(unsigned(2 * n)), 32 * N, smem, s, args, items, active);
+    launch_k(k_apply_fix_batch<N, TS, SPLIT>, dim3(unsigned(SPLIT ? 2 * n : n)), 32 * N, smem, s, args,
+             items, active);
     SIP_CHECK_LAUNCH();
 }
 
@@ -411,16 +418,19 @@ bool launch_apply_fix_list(int N, const OpGeom& g, const float* x, float* y, con
     }
 }
 
+int fix_tile_count(int nx, int ny) { return ((nx + 7) / 8) * ((ny + 3) / 4); }
+
 template <typename TS>
 void launch_apply_fix_batch(int N, const FixArgs<TS>* args, const int2* items, int n_items,
                             const int* active, cudaStream_t s) {
     if (n_items <= 0) return;
+    constexpr bool SPLIT = sizeof(TS) == 4;
     switch (N) {
-        case 2: launch_batch<2, TS>(args, items, n_items, active, s); break;
-        case 3: launch_batch<3, TS>(args, items, n_items, active, s); break;
-        case 4: launch_batch<4, TS>(args, items, n_items, active, s); break;
-        case 5: launch_batch<5, TS>(args, items, n_items, active, s); break;
-        case 6: launch_batch<6, TS>(args, items, n_items, active, s); break;
+        case 2: launch_batch<2, TS, SPLIT>(args, items, n_items, active, s); break;
+        case 3: launch_batch<3, TS, SPLIT>(args, items, n_items, active, s); break;
+        case 4: launch_batch<4, TS, SPLIT>(args, items, n_items, active, s); break;
+        case 5: launch_batch<5, TS, SPLIT>(args, items, n_items, active, s); break;
+        case 6: launch_batch<6, TS, SPLIT>(args, items, n_items, active, s); break;
         default: throw Error(SIP_ERR_INVALID_ARG, "batched apply: degree above 5");
     }
 }

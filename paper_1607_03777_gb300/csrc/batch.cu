@@ -95,33 +95,6 @@ __device__ __forceinline__ double member_sum(const double* partial, int m) {
 
 // ---- element-vector kernels: items (member, chunk of kChunk entries)
 
-// which vector of the p-level a kernel reads / writes
-enum PVec { V_IN, V_OUT, V_PR, V_PD, V_R1, V_E1 };
-template <typename T>
-__device__ __forceinline__ T* pvec(const BMember<T>& b, int v) {
-    switch (v) {
-        case V_IN: return b.vin;
-        case V_OUT: return b.vout;
-        case V_PR: return b.pr;
-        case V_PD: return b.pd;
-        case V_R1: return b.r1;
-        default: return b.e1;
-    }
-}
-
-// dst = src over n_u entries (T)
-template <typename T>
-__global__ void k_b_copy(const BMember<T>* __restrict__ mb, const int2* __restrict__ items,
-                         const int* __restrict__ act, int src, int dst) {
-    grid_dep_wait();
-    const int2 it = items[blockIdx.x];
-    if (!act[it.x]) return;
-    const BMember<T>& b = mb[it.x];
-    const long long g = (long long)it.y * kChunk + threadIdx.x;
-    if (g >= b.n_u) return;
-    pvec(b, dst)[g] = pvec(b, src)[g];
-}
-
 // vin = (T) r   (the V-cycle input, rounded to its precision)
 template <typename T>
 __global__ void k_b_r_to_vin(const BMember<T>* __restrict__ mb, const int2* __restrict__ items,
@@ -133,22 +106,6 @@ __global__ void k_b_r_to_vin(const BMember<T>* __restrict__ mb, const int2* __re
     const long long g = (long long)it.y * kChunk + threadIdx.x;
     if (g >= b.n_u) return;
     b.vin[g] = T(b.r[g]);
-}
-
-// e1 -> y: y += P e1 (hierarchical injection of the Q_1 modes); items over ne * 8
-template <typename T>
-__global__ void k_b_prolong_add(const BMember<T>* __restrict__ mb, const int2* __restrict__ items,
-                                const int* __restrict__ act) {
-    grid_dep_wait();
-    const int2 it = items[blockIdx.x];
-    if (!act[it.x]) return;
-    const BMember<T>& b = mb[it.x];
-    const long long g = (long long)it.y * kChunk + threadIdx.x;
-    if (g >= b.ne * 8) return;
-    const int N = b.N;
-    const long long e = g / 8;
-    const int l = int(g % 8), c = l / 4, j = (l / 2) % 2, i = l % 2;
-    b.vout[e * 2 * N * N + c * N * N + j * N + i] += b.e1[g];
 }
 
 // R_dc: level-0 vertex values from the element Q_1 residual r1; items over hn[0]
@@ -180,9 +137,9 @@ __global__ void k_b_rdc(const BMember<T>* __restrict__ mb, const int2* __restric
     b.hb[0][g] = T(acc);
 }
 
-// P_cd: element Q_1 coefficients e1 from the level-0 vertex values; items over ne * 8
+// y += P P_cd v: the level-0 vertex values' element Q_1 coefficients; items over ne * 8
 template <typename T>
-__global__ void k_b_pcd(const BMember<T>* __restrict__ mb, const int2* __restrict__ items,
+__global__ void k_b_pcd_add(const BMember<T>* __restrict__ mb, const int2* __restrict__ items,
                         const int* __restrict__ act) {
     grid_dep_wait();
     const int2 it = items[blockIdx.x];
@@ -200,7 +157,8 @@ __global__ void k_b_pcd(const BMember<T>* __restrict__ mb, const int2* __restric
         for (int p = 0; p < 2; ++p)
             acc += hatw(i, p) * hatw(j, q) *
                    double(v[2 * ((long long)(ey + q) * (nx + 1) + ex + p) + c]);
-    b.e1[g] = T(acc);
+    const int N = b.N;
+    b.vout[e * 2 * N * N + c * N * N + j * N + i] += T(acc);
 }
 
 // ---- continuous levels: items (member, chunk) over the unknowns of level lv
@@ -617,12 +575,26 @@ struct BatchEngine {
     // arithmetic tiles of split members) and their work lists
     struct Group {
         int N = 0;
-        DeviceBuffer a_dec, a_res, a_r1, a_dec_hi, a_res_hi, a_r1_hi, a_q;
-        DeviceBuffer it_lo, it_hi, it_all, it_bj;
-        int n_lo = 0, n_hi = 0, n_all = 0, n_bj = 0;
+        // operator roles: dec0 pr = vin - A pd (first step from zero), dec pr -= A pd,
+        // res pr = vin - A vout, r1 = R (vin - A vout); staged kernels, and the
+        // fixed-point ones (FP64 operators; the FP64-arithmetic tiles of FP32 ones)
+        DeviceBuffer a[4], a_hi[4], f[4], a_q, f_q;
+        bool fix = false;   // the fixed-point forms apply to every member
+        DeviceBuffer it_lo, it_hi, it_all, it_fix, it_bj;
+        int n_lo = 0, n_hi = 0, n_all = 0, n_fix = 0, n_bj = 0;
         std::vector<DeviceBuffer> bj;   // block-Jacobi tables: [0] first step pre, [1] first step post, [1 + st] step st
     };
     std::vector<Group> groups;
+    // degrees run side by side within a stage: a stream per further group
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> ev;
+    // continuous levels in two launches each (hlevel.cu), where every level allows it
+    struct Level {
+        DeviceBuffer before, after, it_before, it_after;
+        int n_before = 0, n_after = 0, t_before = 0, t_after = 0;
+    };
+    std::vector<Level> levels;
+    bool fused_levels = false;
     // work lists of the vector kernels
     DeviceBuffer it_u, it_parts, it_q1, it_v0, it_coarse;
     int n_u_items = 0, n_parts = 0, n_q1 = 0, n_v0 = 0, n_coarse = 0;
@@ -642,6 +614,21 @@ struct BatchEngine {
         if (graph) cudaGraphDestroy(graph);
         if (cs) cudaStreamDestroy(cs);
         if (pin) cudaFreeHost(pin);
+        for (cudaStream_t t : side) cudaStreamDestroy(t);
+        for (cudaEvent_t t : ev) cudaEventDestroy(t);
+    }
+    // f(group, stream) for every degree: the first on s, the others beside it
+    template <class F>
+    void each_group(cudaStream_t s, F f) {
+        const size_t n = groups.size();
+        if (n > 1) SIP_CUDA(cudaEventRecord(ev[0], s));
+        for (size_t i = 1; i < n; ++i) {
+            SIP_CUDA(cudaStreamWaitEvent(side[i - 1], ev[0], 0));
+            f(groups[i], side[i - 1]);
+            SIP_CUDA(cudaEventRecord(ev[i], side[i - 1]));
+        }
+        if (n > 0) f(groups[0], s);
+        for (size_t i = 1; i < n; ++i) SIP_CUDA(cudaStreamWaitEvent(s, ev[i], 0));
     }
 
     Multigrid<T>& mg(sip_problem* P);
@@ -739,6 +726,42 @@ void BatchEngine<T>::build(cudaStream_t s) {
         n_lv[l] = int(a.size());
         n_lv1[l] = int(b1.size());
     }
+    fused_levels = true;
+    for (int m = 0; m < nmem; ++m)
+        for (int l = 0; l < hm[m].L; ++l)
+            fused_levels = fused_levels && fused_level_ok(mg(probs[m]).h[l], steps_h);
+    levels.clear();
+    if (fused_levels) {
+        levels.resize(max_L);
+        for (int l = 0; l < max_L; ++l) {
+            std::vector<LevelArgs<T>> before(nmem), after(nmem);
+            std::vector<int2> ib, ia;
+            Level& V = levels[l];
+            int n = 0;
+            for (int m = 0; m < nmem; ++m) n += l < hm[m].L ? 1 : 0;
+            for (int m = 0; m < nmem; ++m) {
+                if (l >= hm[m].L) continue;
+                Multigrid<T>& G = mg(probs[m]);
+                HLevel<T>& H = G.h[l];
+                double c1[kMaxSt], c2[kMaxSt];
+                cheb_coefs(probs[m]->desc.cheb_lo * H.lmax, probs[m]->desc.cheb_hi * H.lmax, steps_h, c1, c2);
+                T* x0 = H.d.template as<T>();
+                before[m] = level_before_args<T>(H, G.h[l + 1], steps_h, c1, c2, x0, n);
+                after[m] = level_after_args<T>(H, G.h[l + 1], steps_h, c1, c2, x0, H.x.template as<T>(), n);
+                for (int t = 0; t < before[m].tiles; ++t) ib.push_back({m, t});
+                for (int t = 0; t < after[m].tiles; ++t) ia.push_back({m, t});
+                V.t_before = std::max(V.t_before, before[m].threads);
+                V.t_after = std::max(V.t_after, after[m].threads);
+            }
+            upload(V.before, before, s);
+            upload(V.after, after, s);
+            upload(V.it_before, ib, s);
+            upload(V.it_after, ia, s);
+            V.n_before = int(ib.size());
+            V.n_after = int(ia.size());
+            SIP_CUDA(cudaStreamSynchronize(s));   // staging vectors of this level
+        }
+    }
     upload(d_mem, hm, s);
     upload(it_u, items_u, s);
     upload(it_parts, items_parts, s);
@@ -770,10 +793,18 @@ void BatchEngine<T>::build(cudaStream_t s) {
         if (ms.empty()) continue;
         Group g;
         g.N = N;
-        std::vector<StageArgs<T, T>> dec(nmem), res(nmem), r1(nmem);
-        std::vector<StageArgs<T, double>> dech(nmem), resh(nmem), r1h(nmem);
+        std::vector<StageArgs<T, T>> lo_a[4];
+        std::vector<StageArgs<T, double>> hi_a[4];
+        std::vector<FixArgs<T>> fx[4];
+        for (int r = 0; r < 4; ++r) {
+            lo_a[r].resize(nmem);
+            hi_a[r].resize(nmem);
+            fx[r].resize(nmem);
+        }
         std::vector<StageArgs<double, double>> qa(nmem);
-        std::vector<int2> lo, hi, all, bjit;
+        std::vector<FixArgs<double>> fq(nmem);
+        g.fix = true;
+        std::vector<int2> lo, hi, all, fixed, bjit;
         const int nbj = steps_p + 1;
         std::vector<std::vector<BJBatchArgs<T>>> bjt(nbj, std::vector<BJBatchArgs<T>>(nmem));
         for (int m : ms) {
@@ -784,16 +815,21 @@ void BatchEngine<T>::build(cudaStream_t s) {
                                           : reinterpret_cast<const T*>(P->eta_d.ptr);
             const T* eta_inv = sizeof(T) == 4 ? reinterpret_cast<const T*>(P->eta_inv_f.ptr)
                                               : reinterpret_cast<const T*>(P->eta_inv_d.ptr);
-            dec[m] = stage_args<T, T>(P->geom, b.pd, b.pr, eta, -1.0, b.pr, 1.0, nullptr, N);
-            res[m] = stage_args<T, T>(P->geom, b.vout, b.pr, eta, -1.0, b.vin, 1.0, nullptr, N);
-            r1[m] = stage_args<T, T>(P->geom, b.vout, nullptr, eta, -1.0, b.vin, 1.0, b.r1, N);
-            if constexpr (sizeof(T) == 4) {
-                dech[m] = stage_args<T, double>(P->geom, b.pd, b.pr, eta, -1.0, b.pr, 1.0, nullptr, N);
-                resh[m] = stage_args<T, double>(P->geom, b.vout, b.pr, eta, -1.0, b.vin, 1.0, nullptr, N);
-                r1h[m] = stage_args<T, double>(P->geom, b.vout, nullptr, eta, -1.0, b.vin, 1.0, b.r1, N);
+            const T* in[4] = {b.pd, b.pd, b.vout, b.vout};
+            const T* add[4] = {b.vin, b.pr, b.vin, b.vin};
+            for (int r = 0; r < 4; ++r) {
+                T* out = r == 3 ? nullptr : b.pr;
+                T* out1 = r == 3 ? b.r1 : nullptr;
+                lo_a[r][m] = stage_args<T, T>(P->geom, in[r], out, eta, -1.0, add[r], 1.0, out1, N);
+                if constexpr (sizeof(T) == 4)
+                    hi_a[r][m] = stage_args<T, double>(P->geom, in[r], out, eta, -1.0, add[r], 1.0, out1, N);
+                g.fix = make_fix_args<T>(N, P->geom, in[r], out, eta, -1.0, add[r], 1.0, out1, fx[r][m]) && g.fix;
             }
             qa[m] = stage_args<double, double>(P->geom, b.d, b.q, P->eta_d.template as<double>(), 1.0,
                                                nullptr, 0.0, nullptr, N);
+            g.fix = make_fix_args<double>(N, P->geom, b.d, b.q, P->eta_d.template as<double>(), 1.0,
+                                          nullptr, 0.0, nullptr, fq[m]) && g.fix;
+            for (int t = 0; t < fix_tile_count(b.nx, b.ny); ++t) fixed.push_back({m, t});
             const int nt = split_tile_count(b.nx, b.ny);
             std::vector<unsigned char> flag(size_t(nt), 0);
             if (sizeof(T) == 4 && G.n_hi > 0) {
@@ -812,7 +848,7 @@ void BatchEngine<T>::build(cudaStream_t s) {
                 const int st = k < 2 ? 0 : k - 1;
                 BJBatchArgs<T>& a = bjt[k][m];
                 a.ne = int(b.ne);
-                a.r = b.pr;
+                a.r = k == 0 ? b.vin : b.pr;   // from zero the residual is the input
                 a.out = b.pd;
                 a.x = b.vout;
                 a.emap = G.emap.template as<int>();
@@ -827,13 +863,15 @@ void BatchEngine<T>::build(cudaStream_t s) {
                 a.x_zero = k == 0 ? 1 : 0;
             }
         }
-        upload(g.a_dec, dec, s);
-        upload(g.a_res, res, s);
-        upload(g.a_r1, r1, s);
-        upload(g.a_dec_hi, dech, s);
-        upload(g.a_res_hi, resh, s);
-        upload(g.a_r1_hi, r1h, s);
+        for (int r = 0; r < 4; ++r) {
+            upload(g.a[r], lo_a[r], s);
+            upload(g.a_hi[r], hi_a[r], s);
+            upload(g.f[r], fx[r], s);
+        }
         upload(g.a_q, qa, s);
+        upload(g.f_q, fq, s);
+        upload(g.it_fix, fixed, s);
+        g.n_fix = int(fixed.size());
         upload(g.it_lo, lo, s);
         upload(g.it_hi, hi, s);
         upload(g.it_all, all, s);
@@ -844,7 +882,18 @@ void BatchEngine<T>::build(cudaStream_t s) {
         g.n_bj = int(bjit.size());
         g.bj.resize(nbj);
         for (int k = 0; k < nbj; ++k) upload(g.bj[k], bjt[k], s);
+        SIP_CUDA(cudaStreamSynchronize(s));   // staging vectors of this degree
         groups.push_back(std::move(g));
+    }
+    while (side.size() + 1 < groups.size()) {
+        cudaStream_t t = nullptr;
+        SIP_CUDA(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+        side.push_back(t);
+    }
+    while (ev.size() < groups.size()) {
+        cudaEvent_t t = nullptr;
+        SIP_CUDA(cudaEventCreateWithFlags(&t, cudaEventDisableTiming));
+        ev.push_back(t);
     }
     SIP_CUDA(cudaStreamSynchronize(s));   // host staging vectors are released on return
 }
@@ -853,36 +902,35 @@ template <typename T>
 void BatchEngine<T>::capture_vcycle(cudaStream_t s) {
     const BMember<T>* mb = d_mem.template as<BMember<T>>();
     const int* act = d_act.template as<int>();
-    const int2* iu = it_u.template as<int2>();
-    auto apply = [&](int role) {   // 0: pr -= A pd, 1: pr = vin - A vout, 2: r1 = R(vin - A vout)
-        for (Group& g : groups) {
-            DeviceBuffer& lo = role == 0 ? g.a_dec : (role == 1 ? g.a_res : g.a_r1);
-            DeviceBuffer& hi = role == 0 ? g.a_dec_hi : (role == 1 ? g.a_res_hi : g.a_r1_hi);
-            launch_apply_stage_batch<T, T>(g.N, lo.template as<StageArgs<T, T>>(), g.it_lo.template as<int2>(),
-                                           g.n_lo, act, vec, s);
-            if constexpr (sizeof(T) == 4)
-                launch_apply_stage_batch<T, double>(g.N, hi.template as<StageArgs<T, double>>(),
-                                                    g.it_hi.template as<int2>(), g.n_hi, act, vec, s);
+    auto apply = [&](Group& g, int role, cudaStream_t t) {
+        if constexpr (sizeof(T) == 8) {
+            if (g.fix) {
+                launch_apply_fix_batch<double>(g.N, g.f[role].template as<FixArgs<double>>(),
+                                               g.it_fix.template as<int2>(), g.n_fix, act, t);
+                return;
+            }
+        }
+        launch_apply_stage_batch<T, T>(g.N, g.a[role].template as<StageArgs<T, T>>(),
+                                       g.it_lo.template as<int2>(), g.n_lo, act, vec, t);
+        if constexpr (sizeof(T) == 4) {
+            if (g.fix)
+                launch_apply_fix_batch<float>(g.N, g.f[role].template as<FixArgs<float>>(),
+                                              g.it_hi.template as<int2>(), g.n_hi, act, t);
+            else
+                launch_apply_stage_batch<T, double>(g.N, g.a_hi[role].template as<StageArgs<T, double>>(),
+                                                    g.it_hi.template as<int2>(), g.n_hi, act, vec, t);
         }
     };
-    auto bj = [&](int k) {
-        for (Group& g : groups)
-            launch_bj_apply_batch<T>(g.N, g.bj[k].template as<BJBatchArgs<T>>(), g.it_bj.template as<int2>(), g.n_bj,
-                                     act, s);
+    auto bj = [&](Group& g, int k, cudaStream_t t) {
+        launch_bj_apply_batch<T>(g.N, g.bj[k].template as<BJBatchArgs<T>>(), g.it_bj.template as<int2>(),
+                                 g.n_bj, act, t);
     };
-    auto smooth = [&](bool zero) {
-        if (zero) {
-            launch_k(k_b_copy<T>, dim3(unsigned(n_u_items)), kChunk, 0, s, mb, iu, act, int(V_IN),
-                     int(V_PR));
-            SIP_CHECK_LAUNCH();
-            bj(0);
-        } else {
-            apply(1);
-            bj(1);
-        }
+    auto smooth = [&](Group& g, bool zero, cudaStream_t t) {
+        if (!zero) apply(g, 2, t);
+        bj(g, zero ? 0 : 1, t);
         for (int st = 1; st < steps_p; ++st) {
-            apply(0);
-            bj(1 + st);
+            apply(g, zero && st == 1 ? 0 : 1, t);
+            bj(g, 1 + st, t);
         }
     };
     auto hsmooth = [&](int l, bool zero) {
@@ -900,11 +948,19 @@ void BatchEngine<T>::capture_vcycle(cudaStream_t s) {
     };
     // Algorithm 1: pre-smoothing from y = 0, restricted residual, coarse
     // correction through the continuous levels, prolongation, post-smoothing
-    smooth(true);
-    apply(2);
+    each_group(s, [&](Group& g, cudaStream_t t) {
+        smooth(g, true, t);
+        apply(g, 3, t);
+    });
     launch_k(k_b_rdc<T>, dim3(unsigned(n_v0)), kChunk, 0, s, mb, it_v0.template as<int2>(), act);
     SIP_CHECK_LAUNCH();
     for (int l = 0; l < max_L; ++l) {   // members with l < L go one level down
+        if (fused_levels) {
+            Level& V = levels[l];
+            launch_level_batch<T>(false, V.before.template as<LevelArgs<T>>(), V.it_before.template as<int2>(),
+                                  V.n_before, V.t_before, act, s);
+            continue;
+        }
         hsmooth(l, true);
         launch_k(k_b_hresid<T>, dim3(unsigned(n_lv[l])), kChunk, 0, s, mb, it_lv[l].template as<int2>(),
                  act, l);
@@ -916,16 +972,20 @@ void BatchEngine<T>::capture_vcycle(cudaStream_t s) {
     launch_k(k_b_coarse<T>, dim3(unsigned(n_coarse)), kChunk, 0, s, mb, it_coarse.template as<int2>(), act);
     SIP_CHECK_LAUNCH();
     for (int l = max_L - 1; l >= 0; --l) {
+        if (fused_levels) {
+            Level& V = levels[l];
+            launch_level_batch<T>(true, V.after.template as<LevelArgs<T>>(), V.it_after.template as<int2>(),
+                                  V.n_after, V.t_after, act, s);
+            continue;
+        }
         launch_k(k_b_ph_add<T>, dim3(unsigned(n_lv[l])), kChunk, 0, s, mb, it_lv[l].template as<int2>(),
                  act, l);
         SIP_CHECK_LAUNCH();
         hsmooth(l, false);
     }
-    launch_k(k_b_pcd<T>, dim3(unsigned(n_q1)), kChunk, 0, s, mb, it_q1.template as<int2>(), act);
+    launch_k(k_b_pcd_add<T>, dim3(unsigned(n_q1)), kChunk, 0, s, mb, it_q1.template as<int2>(), act);
     SIP_CHECK_LAUNCH();
-    launch_k(k_b_prolong_add<T>, dim3(unsigned(n_q1)), kChunk, 0, s, mb, it_q1.template as<int2>(), act);
-    SIP_CHECK_LAUNCH();
-    smooth(false);
+    each_group(s, [&](Group& g, cudaStream_t t) { smooth(g, false, t); });
 }
 
 template <typename T>
@@ -950,9 +1010,14 @@ void BatchEngine<T>::capture_body(cudaStream_t s, cudaGraphConditionalHandle h) 
     launch_k(k_b_dir<T>, dim3(unsigned(n_u_items)), kChunk, 0, s, mb,
              static_cast<const BState*>(st), iu, static_cast<const int*>(act));
     SIP_CHECK_LAUNCH();
-    for (Group& g : groups)
-        launch_apply_stage_batch<double, double>(g.N, g.a_q.template as<StageArgs<double, double>>(),
-                                                 g.it_all.template as<int2>(), g.n_all, act, vec, s);
+    each_group(s, [&](Group& g, cudaStream_t t) {
+        if (g.fix)
+            launch_apply_fix_batch<double>(g.N, g.f_q.template as<FixArgs<double>>(),
+                                           g.it_fix.template as<int2>(), g.n_fix, act, t);
+        else
+            launch_apply_stage_batch<double, double>(g.N, g.a_q.template as<StageArgs<double, double>>(),
+                                                     g.it_all.template as<int2>(), g.n_all, act, vec, t);
+    });
     launch_k(k_b_dot_dq<T>, dim3(unsigned(n_parts)), kChunk, 0, s, mb, ip,
              static_cast<const int*>(act), nmem, fl, part);
     SIP_CHECK_LAUNCH();

@@ -20,23 +20,6 @@ namespace sip {
 namespace {
 
 constexpr int kMaxThreads = 768;
-constexpr int kMaxSteps = 4;
-
-template <typename T>
-struct HLevelArgs {
-    int nvx, nvy;     // vertices of this level
-    int ncx, ncy;     // intervals of the next one
-    const T* S;
-    const T* dinv;
-    const T* b;
-    const T* xin;     // after: the iterate before the correction
-    T* x;
-    const T* xc;      // after: coarse correction
-    T* bc;            // before: coarse right-hand side
-    T c1[kMaxSteps], c2[kMaxSteps];
-    int steps, tile, rw;   // coarse vertices of a tile, vertices of its region, per direction
-};
-
 template <typename T>
 __device__ __forceinline__ T row_dot(const T (&s)[18], const T* v, int rw) {
     T acc = T(0);
@@ -68,7 +51,7 @@ struct Place {
 };
 
 template <typename T>
-__device__ __forceinline__ Place place(const HLevelArgs<T>& a, int ox, int oy) {
+__device__ __forceinline__ Place place(const LevelArgs<T>& a, int ox, int oy) {
     Place p;
     p.c = threadIdx.x % 2;
     const int v = threadIdx.x / 2, lx = v % a.rw, ly = v / a.rw;
@@ -83,14 +66,13 @@ __device__ __forceinline__ Place place(const HLevelArgs<T>& a, int ox, int oy) {
 
 // x = Chebyshev steps on S x = b from zero; bc = R_h (b - S x).
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads) k_level_before(const HLevelArgs<T> a) {
-    grid_dep_wait();
+__device__ __forceinline__ void level_before(const LevelArgs<T>& a, int tile) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nt = 2 * a.rw * a.rw;
     T* sd = reinterpret_cast<T*>(smem_raw);   // direction, then iterate
     T* sr = sd + nt;                          // residual
     const int ntx = (a.ncx + a.tile) / a.tile;   // ceil((ncx + 1) / tile)
-    const int I0 = int(blockIdx.x % ntx) * a.tile, J0 = int(blockIdx.x / ntx) * a.tile;
+    const int I0 = (tile % ntx) * a.tile, J0 = (tile / ntx) * a.tile;
     const Place p = place(a, 2 * I0 - 1 - a.steps, 2 * J0 - 1 - a.steps);
     const bool mine = int(threadIdx.x) < nt;
     T s[18], r = T(0), d = T(0), x = T(0), bv = T(0), di = T(0);
@@ -134,13 +116,12 @@ __global__ void __launch_bounds__(kMaxThreads) k_level_before(const HLevelArgs<T
 
 // x = Chebyshev steps on S x = b from xin + P_h xc.
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads) k_level_after(const HLevelArgs<T> a) {
-    grid_dep_wait();
+__device__ __forceinline__ void level_after(const LevelArgs<T>& a, int tile) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nt = 2 * a.rw * a.rw;
     T* sd = reinterpret_cast<T*>(smem_raw);
     const int tf = 2 * a.tile, ntx = (a.nvx + tf - 1) / tf;
-    const int X0 = int(blockIdx.x % ntx) * tf, Y0 = int(blockIdx.x / ntx) * tf;
+    const int X0 = (tile % ntx) * tf, Y0 = (tile / ntx) * tf;
     const Place p = place(a, X0 - a.steps, Y0 - a.steps);
     const bool mine = int(threadIdx.x) < nt;
     T s[18], r = T(0), d = T(0), x = T(0), bv = T(0), di = T(0);
@@ -178,20 +159,40 @@ __global__ void __launch_bounds__(kMaxThreads) k_level_after(const HLevelArgs<T>
     if (p.in && fx >= 0 && fx < tf && fy >= 0 && fy < tf) a.x[p.g] = x;
 }
 
+template <typename T, bool AFTER>
+__global__ void __launch_bounds__(kMaxThreads) k_level(const LevelArgs<T> a) {
+    grid_dep_wait();
+    if constexpr (AFTER) level_after<T>(a, blockIdx.x);
+    else level_before<T>(a, blockIdx.x);
+}
+
+template <typename T, bool AFTER>
+__global__ void __launch_bounds__(kMaxThreads) k_level_batch(const LevelArgs<T>* __restrict__ args,
+                                                             const int2* __restrict__ items,
+                                                             const int* __restrict__ active) {
+    grid_dep_wait();
+    const int2 it = items[blockIdx.x];
+    if (active && !active[it.x]) return;
+    const LevelArgs<T> a = args[it.x];
+    if constexpr (AFTER) level_after<T>(a, it.y);
+    else level_before<T>(a, it.y);
+}
+
 // Coarse vertices per tile and direction: the largest (least recomputation)
 // that still gives most SMs a tile.
-int level_tile(int nvxc, int nvyc, int steps) {
+int level_tile(int nvxc, int nvyc, int steps, int members) {
     for (int t = 6; t > 2; --t) {
         const int rw = 2 * t + 1 + 2 * steps;
         if (2 * rw * rw > kMaxThreads) continue;
-        if (((nvxc + t - 1) / t) * ((nvyc + t - 1) / t) >= 110) return t;
+        if (((nvxc + t - 1) / t) * ((nvyc + t - 1) / t) * members >= 110) return t;
     }
     return 2;
 }
 
 template <typename T>
-HLevelArgs<T> level_args(const HLevel<T>& L, const HLevel<T>& C, int steps, const T* c1, const T* c2) {
-    HLevelArgs<T> a{};
+LevelArgs<T> level_args(const HLevel<T>& L, const HLevel<T>& C, int steps, const double* c1,
+                        const double* c2, T* x, int members) {
+    LevelArgs<T> a{};
     a.nvx = L.nvx;
     a.nvy = L.nvy;
     a.ncx = C.nx;
@@ -199,62 +200,83 @@ HLevelArgs<T> level_args(const HLevel<T>& L, const HLevel<T>& C, int steps, cons
     a.S = L.S.template as<T>();
     a.dinv = L.dinv.template as<T>();
     a.b = L.b.template as<T>();
+    a.x = x;
     a.steps = steps;
-    a.tile = level_tile(C.nvx, C.nvy, steps);
+    a.tile = level_tile(C.nvx, C.nvy, steps, members);
     for (int i = 0; i < steps; ++i) {
-        a.c1[i] = c1[i];
-        a.c2[i] = c2[i];
+        a.c1[i] = T(c1[i]);
+        a.c2[i] = T(c2[i]);
     }
     return a;
 }
 
-inline unsigned round32(int n) { return unsigned((n + 31) / 32 * 32); }
+inline int round32(int n) { return (n + 31) / 32 * 32; }
 
 }  // namespace
 
 template <typename T>
 bool fused_level_ok(const HLevel<T>& L, int steps) {
-    if (steps < 1 || steps > kMaxSteps) return false;
-    const int rw = 2 * 2 + 1 + 2 * steps;
-    if (2 * rw * rw > kMaxThreads) return false;
+    if (steps < 1 || steps > kLevelSteps) return false;
     return sizeof(T) == 4 || size_t(L.nvx) * L.nvy <= size_t(300) * 300;
 }
-template bool fused_level_ok<float>(const HLevel<float>&, int);
-template bool fused_level_ok<double>(const HLevel<double>&, int);
 
 template <typename T>
-void launch_level_before(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, T* x,
-                         cudaStream_t s) {
-    HLevelArgs<T> a = level_args(L, C, steps, c1, c2);
+LevelArgs<T> level_before_args(HLevel<T>& L, HLevel<T>& C, int steps, const double* c1, const double* c2,
+                               T* x, int members) {
+    LevelArgs<T> a = level_args(L, C, steps, c1, c2, x, members);
     a.rw = 2 * a.tile + 1 + 2 * steps;
-    a.x = x;
     a.bc = C.b.template as<T>();
-    const int nt = 2 * a.rw * a.rw, t = a.tile;
-    const unsigned grid = unsigned(((C.nvx + t - 1) / t) * ((C.nvy + t - 1) / t));
-    launch_k(k_level_before<T>, grid, round32(nt), size_t(2 * nt) * sizeof(T), s, a);
-    SIP_CHECK_LAUNCH();
+    a.tiles = ((C.nvx + a.tile - 1) / a.tile) * ((C.nvy + a.tile - 1) / a.tile);
+    a.threads = round32(2 * a.rw * a.rw);
+    return a;
 }
-template void launch_level_before<float>(HLevel<float>&, HLevel<float>&, int, const float*, const float*,
-                                         float*, cudaStream_t);
-template void launch_level_before<double>(HLevel<double>&, HLevel<double>&, int, const double*,
-                                          const double*, double*, cudaStream_t);
 
 template <typename T>
-void launch_level_after(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, const T* xin,
-                        T* x, cudaStream_t s) {
-    HLevelArgs<T> a = level_args(L, C, steps, c1, c2);
-    a.rw = 2 * a.tile + 2 * steps;
+LevelArgs<T> level_after_args(HLevel<T>& L, HLevel<T>& C, int steps, const double* c1, const double* c2,
+                              const T* xin, T* x, int members) {
+    LevelArgs<T> a = level_args(L, C, steps, c1, c2, x, members);
+    const int tf = 2 * a.tile;
+    a.rw = tf + 2 * steps;
     a.xin = xin;
-    a.x = x;
     a.xc = C.x.template as<T>();
-    const int nt = 2 * a.rw * a.rw, tf = 2 * a.tile;
-    const unsigned grid = unsigned(((L.nvx + tf - 1) / tf) * ((L.nvy + tf - 1) / tf));
-    launch_k(k_level_after<T>, grid, round32(nt), size_t(nt) * sizeof(T), s, a);
+    a.tiles = ((L.nvx + tf - 1) / tf) * ((L.nvy + tf - 1) / tf);
+    a.threads = round32(2 * a.rw * a.rw);
+    return a;
+}
+
+template <typename T>
+void launch_level(const LevelArgs<T>& a, cudaStream_t s) {
+    const size_t smem = size_t(2) * a.threads * sizeof(T);   // two vectors of a tile's region
+    if (a.xin)
+        launch_k(k_level<T, true>, unsigned(a.tiles), unsigned(a.threads), smem, s, a);
+    else
+        launch_k(k_level<T, false>, unsigned(a.tiles), unsigned(a.threads), smem, s, a);
     SIP_CHECK_LAUNCH();
 }
-template void launch_level_after<float>(HLevel<float>&, HLevel<float>&, int, const float*, const float*,
-                                        const float*, float*, cudaStream_t);
-template void launch_level_after<double>(HLevel<double>&, HLevel<double>&, int, const double*,
-                                         const double*, const double*, double*, cudaStream_t);
+
+template <typename T>
+void launch_level_batch(bool after, const LevelArgs<T>* args, const int2* items, int n_items, int threads,
+                        const int* active, cudaStream_t s) {
+    if (n_items <= 0) return;
+    const size_t smem = size_t(2) * threads * sizeof(T);
+    if (after)
+        launch_k(k_level_batch<T, true>, unsigned(n_items), unsigned(threads), smem, s, args, items, active);
+    else
+        launch_k(k_level_batch<T, false>, unsigned(n_items), unsigned(threads), smem, s, args, items, active);
+    SIP_CHECK_LAUNCH();
+}
+
+#define SIP_LEVEL(T)                                                                              \
+    template bool fused_level_ok<T>(const HLevel<T>&, int);                                       \
+    template LevelArgs<T> level_before_args<T>(HLevel<T>&, HLevel<T>&, int, const double*,        \
+                                               const double*, T*, int);                           \
+    template LevelArgs<T> level_after_args<T>(HLevel<T>&, HLevel<T>&, int, const double*,         \
+                                              const double*, const T*, T*, int);                  \
+    template void launch_level<T>(const LevelArgs<T>&, cudaStream_t);                             \
+    template void launch_level_batch<T>(bool, const LevelArgs<T>*, const int2*, int, int, const int*, \
+                                        cudaStream_t);
+SIP_LEVEL(double)
+SIP_LEVEL(float)
+#undef SIP_LEVEL
 
 }  // namespace sip

@@ -100,7 +100,9 @@ struct FixArgs {
 template <typename TS>
 bool make_fix_args(int N, const OpGeom& g, const TS* x, TS* y, const TS* eta, double alpha, const TS* z,
                    double beta, TS* r1, FixArgs<TS>& a);
-// items: (member, 32 x 2 tile); active (may be null) masks members
+// items: (member, tile of fix_tile_count) for FP64 vectors, (member, 32 x 2
+// split-precision tile) for FP32; active (may be null) masks members
+int fix_tile_count(int nx, int ny);
 template <typename TS>
 void launch_apply_fix_batch(int N, const FixArgs<TS>* args, const int2* items, int n_items,
                             const int* active, cudaStream_t s);

@@ -133,13 +133,36 @@ struct HLevel {
 // ---- hlevel.cu: a level's work before and after its coarse correction, one
 // launch each (Chebyshev coefficients c1, c2 per step; x, xin: iterate buffers
 // that differ).  fused_level_ok: number of steps and level size it serves.
+constexpr int kLevelSteps = 4;
+template <typename T>
+struct LevelArgs {
+    int nvx, nvy;     // vertices of this level
+    int ncx, ncy;     // intervals of the next one
+    const T* S;
+    const T* dinv;
+    const T* b;
+    const T* xin;     // after: the iterate before the correction
+    T* x;
+    const T* xc;      // after: coarse correction
+    T* bc;            // before: coarse right-hand side
+    T c1[kLevelSteps], c2[kLevelSteps];
+    int steps, tile, rw;   // coarse vertices of a tile, vertices of its region, per direction
+    int tiles, threads;    // CTAs and threads per CTA
+};
 template <typename T> bool fused_level_ok(const HLevel<T>& L, int steps);
+// members: number of levels that share the launch (more members, larger tiles)
 template <typename T>
-void launch_level_before(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, T* x,
-                         cudaStream_t s);
+LevelArgs<T> level_before_args(HLevel<T>& L, HLevel<T>& C, int steps, const double* c1, const double* c2,
+                               T* x, int members = 1);
 template <typename T>
-void launch_level_after(HLevel<T>& L, HLevel<T>& C, int steps, const T* c1, const T* c2, const T* xin,
-                        T* x, cudaStream_t s);
+LevelArgs<T> level_after_args(HLevel<T>& L, HLevel<T>& C, int steps, const double* c1, const double* c2,
+                              const T* xin, T* x, int members = 1);
+template <typename T> void launch_level(const LevelArgs<T>& a, cudaStream_t s);   // xin null: before
+// Many levels in one launch: items (member, tile), members with active[m] == 0
+// skipped; threads: the largest of the members'
+template <typename T>
+void launch_level_batch(bool after, const LevelArgs<T>* args, const int2* items, int n_items, int threads,
+                        const int* active, cudaStream_t s);
 
 template <typename T>
 struct Multigrid {

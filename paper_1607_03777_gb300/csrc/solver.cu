@@ -811,20 +811,20 @@ void Multigrid<T>::hcycle(int l, cudaStream_t s) {
     const int steps = P->desc.cheb_steps_h;
     if (fused_level_ok(Lv, steps)) {
         const Cheb ch(P->desc.cheb_lo * Lv.lmax, P->desc.cheb_hi * Lv.lmax);
-        std::vector<T> c1(steps), c2(steps);
-        c1[0] = T(0);
-        c2[0] = T(1.0 / ch.theta);
+        double c1[kLevelSteps], c2[kLevelSteps];
+        c1[0] = 0.0;
+        c2[0] = 1.0 / ch.theta;
         double rho = 1.0 / ch.sigma;
         for (int st = 1; st < steps; ++st) {
             const double rn = 1.0 / (2.0 * ch.sigma - rho);
-            c1[st] = T(rn * rho);
-            c2[st] = T(2.0 * rn / ch.delta);
+            c1[st] = rn * rho;
+            c2[st] = 2.0 * rn / ch.delta;
             rho = rn;
         }
         T* x0 = Lv.d.template as<T>();
-        launch_level_before<T>(Lv, C, steps, c1.data(), c2.data(), x0, s);
+        launch_level<T>(level_before_args<T>(Lv, C, steps, c1, c2, x0), s);
         hcycle(l + 1, s);
-        launch_level_after<T>(Lv, C, steps, c1.data(), c2.data(), x0, Lv.x.template as<T>(), s);
+        launch_level<T>(level_after_args<T>(Lv, C, steps, c1, c2, x0, Lv.x.template as<T>()), s);
         return;
     }
     smooth_h(l, true, s);
