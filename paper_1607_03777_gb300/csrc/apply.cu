@@ -301,7 +301,7 @@ struct BArgs {
     Tab1D<N, T> tab;
 };
 
-// Double-double instances (FP64: apply_div.cu).
+// Double-double, and FP64 where the schedule asks for it (else apply_div.cu).
 // B p: one thread per velocity output (e, c, jq, iq); N = k + 1, pressure
 // degree k - 1 (indices < K = N - 1).
 template <int N, typename T>
@@ -499,7 +499,7 @@ void launch_apply_sip(int N, const OpGeom& g, const T* x, T* y, const T* eta, T 
             return;
     }
     // the FP64 operator's default is the staged entry too (fixed-point kernel)
-    if ((v == APPLY_STAGE || split || (sizeof(T) == 8 && v == APPLY_AUTO)) &&
+    if ((v == APPLY_STAGE || split || (sizeof(T) == 8 && v == APPLY_AUTO && !g.fp64)) &&
         launch_apply_sip_stage<T>(N, g, x, y, eta, alpha, z, beta, nullptr, s))
         return;
     if constexpr (sizeof(T) == 4) {
@@ -538,7 +538,7 @@ template void launch_apply_sip<float>(int, const OpGeom&, const float*, float*, 
                                       float, const float*, float, cudaStream_t);
 
 template <typename T>
-void launch_apply_B(int k, const OpGeom& g, const T* p, T* y, cudaStream_t s) {
+void launch_apply_B_modes(int k, const OpGeom& g, const T* p, T* y, cudaStream_t s) {
     const size_t total = size_t(g.nx) * g.ny * 2 * (k + 1) * (k + 1);
     const unsigned blocks = unsigned((total + 255) / 256);
     switch (k + 1) {
@@ -552,7 +552,7 @@ void launch_apply_B(int k, const OpGeom& g, const T* p, T* y, cudaStream_t s) {
 }
 
 template <typename T>
-void launch_apply_Bt(int k, const OpGeom& g, const T* u, T* y, cudaStream_t s) {
+void launch_apply_Bt_modes(int k, const OpGeom& g, const T* u, T* y, cudaStream_t s) {
     const size_t total = size_t(g.nx) * g.ny * k * k;
     const unsigned blocks = unsigned((total + 255) / 256);
     switch (k + 1) {
@@ -581,8 +581,16 @@ void launch_apply_sip_dd(int N, const OpGeom& g, const dd* x, dd* y, const dd* e
         default: throw Error(SIP_ERR_INVALID_ARG, "unsupported polynomial degree");
     }
 }
-template void launch_apply_B<dd>(int, const OpGeom&, const dd*, dd*, cudaStream_t);
-template void launch_apply_Bt<dd>(int, const OpGeom&, const dd*, dd*, cudaStream_t);
+template <>
+void launch_apply_B<dd>(int k, const OpGeom& g, const dd* p, dd* y, cudaStream_t s) {
+    launch_apply_B_modes<dd>(k, g, p, y, s);
+}
+template <>
+void launch_apply_Bt<dd>(int k, const OpGeom& g, const dd* u, dd* y, cudaStream_t s) {
+    launch_apply_Bt_modes<dd>(k, g, u, y, s);
+}
+template void launch_apply_B_modes<double>(int, const OpGeom&, const double*, double*, cudaStream_t);
+template void launch_apply_Bt_modes<double>(int, const OpGeom&, const double*, double*, cudaStream_t);
 
 void launch_rhs_body_force(int k, const OpGeom& g, const double* rho, double grav, double* f,
                            cudaStream_t s) {

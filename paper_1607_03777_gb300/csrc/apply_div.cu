@@ -198,11 +198,13 @@ void launch_div_k(int k, const OpGeom& g, const double* in, double* out, cudaStr
 
 template <>
 void launch_apply_B<double>(int k, const OpGeom& g, const double* p, double* y, cudaStream_t s) {
-    launch_div_k<false>(k, g, p, y, s);
+    if (g.fp64) launch_apply_B_modes<double>(k, g, p, y, s);
+    else launch_div_k<false>(k, g, p, y, s);
 }
 template <>
 void launch_apply_Bt<double>(int k, const OpGeom& g, const double* u, double* y, cudaStream_t s) {
-    launch_div_k<true>(k, g, u, y, s);
+    if (g.fp64) launch_apply_Bt_modes<double>(k, g, u, y, s);
+    else launch_div_k<true>(k, g, u, y, s);
 }
 
 }  // namespace sip

@@ -1,5 +1,6 @@
 // SIP apply with FP64-accurate results in 64-bit fixed point (fix_core.cuh):
-// the FP64 operator for k <= 5, and the part of the FP32 operator that needs
+// the FP64 operator for k <= 5 (but for Stokes solves of stiff problems: geom_solve in
+// sip_solver.h), and the part of the FP32 operator that needs
 // FP64 arithmetic (split precision: FP32 storage, the tiles of hi_tiles).
 //
 // What bounds it: the integer pipes (about 4000 wide multiply-adds and

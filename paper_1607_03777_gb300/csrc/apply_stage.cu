@@ -541,7 +541,7 @@ void stage_dispatch(const OpGeom& g, const T* x, T* y, const T* eta, T alpha, co
         }
     } else {
         // FP64: the fixed-point kernel wherever it applies
-        if (launch_apply_fix(N, g, x, y, eta, alpha, z, beta, r1, s)) return;
+        if (!g.fp64 && launch_apply_fix(N, g, x, y, eta, alpha, z, beta, r1, s)) return;
     }
     if constexpr (StageLayout<N, T, T, 4>::BYTES <= kMaxSmem) {
         if (g.stage_rows[sizeof(T) == 4 ? 1 : 0] == 4) {

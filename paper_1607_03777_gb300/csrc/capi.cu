@@ -183,6 +183,8 @@ sip_status sip_problem_create(sip_ctx* ctx, const sip_problem_desc* d, sip_probl
             p->n_u = ne * p->nb;
             p->n_p = ne * p->mp;
             p->geom = sip::make_geom(d->nx, d->ny, d->lx, d->ly, d->bc, d->k, d->penalty_scale);
+            p->geom_solve = p->geom;
+            p->geom_solve.fp64 = 1;
             p->geom1 = p->geom;   // the Galerkin A_1 keeps the fine-k penalty
             // continuous vectors, whose jumps cancel exactly in FP64 arithmetic: the
             // coarse problem is nearly singular where a stiff inclusion floats, and
@@ -255,13 +257,15 @@ sip_status sip_problem_set_schedule(sip_problem* p, const int apply[2], const in
         if (apply) {
             p->pin_apply[t] = apply[t];
             if (apply[t] > 0) {
-                p->geom.variant[t] = apply[t] == 5 ? int(sip::APPLY_STAGE) : apply[t];
-                p->geom.stage_rows[t] = apply[t] == 5 ? 4 : 2;
+                for (sip::OpGeom* g : {&p->geom, &p->geom_solve}) {
+                    g->variant[t] = apply[t] == 5 ? int(sip::APPLY_STAGE) : apply[t];
+                    g->stage_rows[t] = apply[t] == 5 ? 4 : 2;
+                }
             }
         }
         if (fused) {
             p->pin_fused[t] = fused[t];
-            if (fused[t] >= 0) p->geom.fused[t] = fused[t];
+            if (fused[t] >= 0) p->geom.fused[t] = p->geom_solve.fused[t] = fused[t];
         }
     }
     // the captured V-cycles hold the old kernels: rebuild at the next use
@@ -292,6 +296,7 @@ sip_status sip_problem_update_eta(sip_problem* p, const double* eta, void* strea
         if (on_dev && !sip::eta_valid(ne, p->eta_d.as<double>(), s))
             throw Error(SIP_ERR_INVALID_ARG, "eta must be finite and positive");
         p->derive_eta(s);
+        p->contrast_known = false;
         if (p->mg64) p->mg64->ready = false;
         if (p->mg32) p->mg32->ready = false;
         if (p->ws) p->ws->sinv_ready = false;

@@ -545,7 +545,7 @@ void capture_body(sip_problem* P, Workspace& W, InnerLoop& L, cudaGraphCondition
     SIP_CHECK_LAUNCH();
     launch_k(k_dir, nblk(n_u), 256, 0, cs, n_u, z, d, st);
     SIP_CHECK_LAUNCH();
-    launch_apply_sip<double>(P->n, P->geom, d, q, P->eta_d.as<double>(), 1.0, nullptr, 0.0, cs);
+    launch_apply_sip<double>(P->n, P->op(), d, q, P->eta_d.as<double>(), 1.0, nullptr, 0.0, cs);
     if (L.flexible) {
         launch_k(k_dot_dq_dr, kRB, kRT, 0, cs, n_u, d, q, r, part);
         SIP_CHECK_LAUNCH();
@@ -596,7 +596,7 @@ void capture_body_pnorm(sip_problem* P, Workspace& W, InnerLoop& L, cudaGraphCon
     PcgState* st = L.state.as<PcgState>();
     launch_k(k_dir, nblk(n_u), 256, 0, cs, n_u, z, d, st);
     SIP_CHECK_LAUNCH();
-    launch_apply_sip<double>(P->n, P->geom, d, q, P->eta_d.as<double>(), 1.0, nullptr, 0.0, cs);
+    launch_apply_sip<double>(P->n, P->op(), d, q, P->eta_d.as<double>(), 1.0, nullptr, 0.0, cs);
     if (L.flexible) {
         launch_k(k_dot_dq_dr, kRB, kRT, 0, cs, n_u, d, q, r, part);
         SIP_CHECK_LAUNCH();
@@ -637,7 +637,7 @@ void capture_body_gcr(sip_problem* P, Workspace& W, InnerLoop& L, cudaGraphCondi
     } else {
         P->mg64->vcycle_on(r, z, cs);
     }
-    launch_apply_sip<double>(P->n, P->geom, z, q, P->eta_d.as<double>(), 1.0, nullptr, 0.0, cs);
+    launch_apply_sip<double>(P->n, P->op(), z, q, P->eta_d.as<double>(), 1.0, nullptr, 0.0, cs);
     for (int pass = 0; pass < 2; ++pass) {
         const bool first = pass == 0;
         launch_k(k_gcr_mdot, kRB, kRT, 0, cs, n_u, first ? static_cast<const double*>(q) : nullptr,
@@ -759,8 +759,9 @@ int inner_pcg_graph(sip_problem* P, Workspace& W, bool mixed, bool flexible, boo
     maxit = std::max(1, std::min(maxit, 100000));
     const size_t n_u = size_t(P->n_u);
     for (DeviceBuffer* b : {&W.cg_r, &W.cg_d, &W.cg_q, &W.cg_z}) b->alloc(n_u * sizeof(double));
-    if (!W.loop) W.loop.reset(new InnerLoop());
-    InnerLoop& L = *W.loop;
+    auto& slot = W.loop[P->in_stokes ? 1 : 0];   // one graph per schedule
+    if (!slot) slot.reset(new InnerLoop());
+    InnerLoop& L = *slot;
     static_assert(sizeof(PcgState) <= 256 * sizeof(double), "state fits the pinned block");
     if (gcr_restart < 0 || gcr_restart > kGcrMax) throw Error(SIP_ERR_INVALID_ARG, "GCR restart");
     L.state.alloc(sizeof(PcgState));

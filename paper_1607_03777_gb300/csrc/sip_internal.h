@@ -160,6 +160,7 @@ struct OpGeom {
     int variant[2];   // ApplyVariant (APPLY_AUTO: component-split for N <= 6, else tile)
     int fused[2];     // p-level smoother step fused into one launch (1) or not (0)
     int stage_rows[2];   // tile rows of the staged apply (2 or 4), per precision
+    int fp64;   // 1: the FP64 operator, B and B^T in FP64 arithmetic throughout (solve_geom)
     // split-precision FP32 operator (mixed form at high viscosity contrast):
     // tiles evaluated in FP64 arithmetic on FP32 data; n_hi = 0: none
     const unsigned char* hi_flag;
@@ -179,6 +180,7 @@ inline OpGeom make_geom(int nx, int ny, double lx, double ly, const int bc[4], i
     g.variant[0] = g.variant[1] = APPLY_AUTO;
     g.fused[0] = g.fused[1] = 1;
     g.stage_rows[0] = g.stage_rows[1] = 2;
+    g.fp64 = 0;
     g.hi_flag = nullptr;
     g.hi_tiles = nullptr;
     g.n_hi = 0;
@@ -248,7 +250,12 @@ template <typename T>
 void launch_apply_B(int k, const OpGeom& g, const T* p, T* y, cudaStream_t s);
 template <typename T>
 void launch_apply_Bt(int k, const OpGeom& g, const T* u, T* y, cudaStream_t s);
-// FP64: apply_div.cu; double-double: apply.cu
+// FP64: apply_div.cu, or with g.fp64 the one-thread-per-mode kernels
+// (launch_apply_B_modes) of apply.cu; double-double: apply.cu
+template <typename T>
+void launch_apply_B_modes(int k, const OpGeom& g, const T* p, T* y, cudaStream_t s);
+template <typename T>
+void launch_apply_Bt_modes(int k, const OpGeom& g, const T* u, T* y, cudaStream_t s);
 template <>
 void launch_apply_B<double>(int k, const OpGeom& g, const double* p, double* y, cudaStream_t s);
 template <>

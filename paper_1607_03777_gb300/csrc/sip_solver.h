@@ -215,6 +215,7 @@ struct Multigrid {
     void hlevel_apply(int l, const T* x, T* y, cudaStream_t s);
     // choose fused or split p-level smoother steps by timing (tune.cu)
     void tune_smoother(cudaStream_t s);
+    void tune_smoother(OpGeom& g, cudaStream_t s);
     int inner_pcg(const T* t, T* y, double rtol, int maxit, cudaStream_t s, double* final_rel);
     int64_t bytes() const;
 
@@ -249,7 +250,7 @@ struct Workspace {
     DeviceBuffer gcr_z, gcr_q;                    // inner GCR directions [m][n_u] each
     DeviceBuffer t32, y32;                        // FP32 inner PCG (SIP_PREC_MIXED_F32_INNER)
     HostScalars hs, hs_in;
-    std::unique_ptr<InnerLoop, InnerLoopDeleter> loop;
+    std::unique_ptr<InnerLoop, InnerLoopDeleter> loop[2];   // viscous solves; Stokes solves in FP64
     bool sinv_ready = false;
     int64_t bytes() const;
 };
@@ -325,11 +326,29 @@ struct sip_problem {
     int k = 0, n = 0, nb = 0, mp = 0;
     int64_t ne = 0, n_u = 0, n_p = 0;
     sip::OpGeom geom{};      // the SIP operator of degree k
+    // Schedule of a Stokes solve whose viscosity contrast is above kFixedContrast:
+    // FP64 arithmetic in every operator.  There the saddle system's attainable
+    // residual in FP64 comes near the tolerances in use (3e-9 of ||b|| for a stiff
+    // box of contrast 1e4 at 128^2, k = 3); a solve whose true residual misses the
+    // tolerance when its recurrence meets it continues from rounding errors, and the
+    // solution then depends on the operators' last bits by 1e-9 to 5e-7 of its norm.
+    // Below, two roundings of the operators agree to 1e-11 after a solve (40 x 32 to
+    // 80 x 64, k = 2 to 4, contrast 19 to 170).  128^2, k = 3, contrast 1e4: 137 ms a step,
+    // 101 ms with the fixed-point operator.
+    sip::OpGeom geom_solve{};
+    static constexpr double kFixedContrast = 128.0;
+    sip::DeviceBuffer eta_range;   // bits of the smallest and largest viscosity
+    bool stiff = false;            // contrast above kFixedContrast
+    bool contrast_known = false;   // stiff belongs to the present viscosities
+    bool in_stokes = false;        // a stiff problem's Stokes solve is running
+    const sip::OpGeom& op() const { return in_stokes ? geom_solve : geom; }
     sip::OpGeom geom1{};     // the Galerkin Q_1 operator (fine-k penalty)
     std::vector<double> eta_host;
     sip::DeviceBuffer eta_d, eta_f, eta_inv_d, eta_inv_f;
     // refresh the FP32 copy and the FP64 / FP32 reciprocals of eta_d
     void derive_eta(cudaStream_t s);
+    // set stiff from the viscosities (once per update of them; synchronises s)
+    void find_contrast(cudaStream_t s);
     std::unique_ptr<sip::Multigrid<double>> mg64;
     std::unique_ptr<sip::Multigrid<float>> mg32;
     std::unique_ptr<sip::Workspace> ws;

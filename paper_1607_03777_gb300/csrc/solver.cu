@@ -398,10 +398,12 @@ double Multigrid<T>::estimate_p(cudaStream_t s) {
     launch_splitmix_uniform(n_u, P->desc.seed, b64.as<double>(), s);
     launch_cast<double, T>(n_u, b64.as<double>(), tmp.template as<T>(), s);
     bj(tmp.template as<T>(), Vp, s);
+    // both schedules share the bound: estimated with the one that is held to FP64
+    const OpGeom& g = P->stiff ? P->geom_solve : P->geom;
     return arnoldi_lmax<T>(n_u, m, Vp, scr_t2, ws.as<double>(), hs,
                            [&](const T* v, T* w) {
-                               launch_apply_sip<T>(N, P->geom, v, tmp.template as<T>(), eta_of<T>(P),
-                                                   T(1), nullptr, T(0), s);
+                               launch_apply_sip<T>(N, g, v, tmp.template as<T>(), eta_of<T>(P), T(1),
+                                                   nullptr, T(0), s);
                                bj(tmp.template as<T>(), w, s);
                            },
                            s);
@@ -478,20 +480,22 @@ void Multigrid<T>::mark_split_tiles(cudaStream_t s) {
         }
     }
     if (sizeof(T) == 4) {
-        P->geom.n_hi = n_hi;
-        P->geom.hi_flag = n_hi > 0 ? hi_flag.as<unsigned char>() : nullptr;
-        P->geom.hi_tiles = n_hi > 0 ? hi_list.as<int>() : nullptr;
+        for (OpGeom* g : {&P->geom, &P->geom_solve}) {
+            g->n_hi = n_hi;
+            g->hi_flag = n_hi > 0 ? hi_flag.as<unsigned char>() : nullptr;
+            g->hi_tiles = n_hi > 0 ? hi_list.as<int>() : nullptr;
+        }
     }
 }
 
 template <typename T>
 bool Multigrid<T>::residual_restrict(const T* y, const T* b, T* r1, cudaStream_t s) {
-    const bool split = sizeof(T) == 4 && P->geom.n_hi > 0;
-    const int v = apply_variant<T>(P->geom);
-    if (split || v == APPLY_STAGE || (sizeof(T) == 8 && v == APPLY_AUTO))
-        return launch_apply_sip_stage<T>(N, P->geom, y, nullptr, eta_of<T>(P), T(-1), b, T(1), r1,
+    const bool split = sizeof(T) == 4 && P->op().n_hi > 0;
+    const int v = apply_variant<T>(P->op());
+    if (split || v == APPLY_STAGE || (sizeof(T) == 8 && v == APPLY_AUTO && !P->op().fp64))
+        return launch_apply_sip_stage<T>(N, P->op(), y, nullptr, eta_of<T>(P), T(-1), b, T(1), r1,
                                          s);
-    return use_fused() && launch_residual_restrict_elem<T>(N, P->geom, y, b, eta_of<T>(P), r1, s);
+    return use_fused() && launch_residual_restrict_elem<T>(N, P->op(), y, b, eta_of<T>(P), r1, s);
 }
 
 template <typename T>
@@ -515,6 +519,7 @@ void Multigrid<T>::setup(cudaStream_t s) {
     cg_r.alloc(n_u * sizeof(T));
     cg_d.alloc(n_u * sizeof(T));
     cg_q.alloc(n_u * sizeof(T));
+    P->find_contrast(s);
     build_blocks(s);
     mark_split_tiles(s);
     lmax_p = estimate_p(s);
@@ -698,9 +703,9 @@ bool Multigrid<T>::use_fused() const {
     }();
     if (env_off || !pd2.ptr || !cheb_elem_available(N)) return false;
     // the fused step evaluates the operator in T everywhere
-    if (sizeof(T) == 4 && P->geom.n_hi > 0) return false;
+    if (sizeof(T) == 4 && P->op().n_hi > 0) return false;
     if (forced >= 0) return forced == 1;
-    return P->geom.fused[sizeof(T) == 4 ? 1 : 0] != 0;
+    return P->op().fused[sizeof(T) == 4 ? 1 : 0] != 0;
 }
 
 template <typename T>
@@ -729,7 +734,7 @@ void Multigrid<T>::smooth_p(const T* b, T* y, bool zero, cudaStream_t s) {
             launch_bj_apply<T>(N, int(ne), b, dA, y, em, ci, cs, ui, einv0, T(0), T(1.0 / ch.theta),
                                true, s, bj_hi(), bj_inv64());
         } else {
-            launch_cheb_elem<T>(N, P->geom, y, b, r, eta, em, ci, cs, ui, einv0, nullptr, dA, nullptr,
+            launch_cheb_elem<T>(N, P->op(), y, b, r, eta, em, ci, cs, ui, einv0, nullptr, dA, nullptr,
                                 T(0), T(1.0 / ch.theta), false, s);
             pend = true;
         }
@@ -737,7 +742,7 @@ void Multigrid<T>::smooth_p(const T* b, T* y, bool zero, cudaStream_t s) {
         double rho = 1.0 / ch.sigma;
         for (int st = 1; st < steps; ++st) {
             const double rn = 1.0 / (2.0 * ch.sigma - rho);
-            launch_cheb_elem<T>(N, P->geom, dA, zsrc, r, eta, em, ci, cs, ui, einv0, dA, dB, y,
+            launch_cheb_elem<T>(N, P->op(), dA, zsrc, r, eta, em, ci, cs, ui, einv0, dA, dB, y,
                                 T(rn * rho), T(2.0 * rn / ch.delta), pend, s);
             pend = false;
             std::swap(dA, dB);
@@ -747,7 +752,7 @@ void Multigrid<T>::smooth_p(const T* b, T* y, bool zero, cudaStream_t s) {
         return;
     }
     // from zero the first residual is b itself: read where it lies
-    if (!zero) launch_apply_sip<T>(N, P->geom, y, r, eta, T(-1), b, T(1), s);   // r = b - A y
+    if (!zero) launch_apply_sip<T>(N, P->op(), y, r, eta, T(-1), b, T(1), s);   // r = b - A y
     const T* r0 = zero ? b : r;
     double rho = 1.0 / ch.sigma;
     const T* einv = eta_inv_of<T>(P);
@@ -755,7 +760,7 @@ void Multigrid<T>::smooth_p(const T* b, T* y, bool zero, cudaStream_t s) {
                        cls_sym.as<int>(), uniq_inv.template as<T>(), einv,
                        T(0), T(1.0 / ch.theta), zero, s, bj_hi(), bj_inv64());
     for (int st = 1; st < P->desc.cheb_steps_p; ++st) {
-        launch_apply_sip<T>(N, P->geom, dd, r, eta, T(-1), st == 1 ? r0 : r, T(1), s);  // r -= A d
+        launch_apply_sip<T>(N, P->op(), dd, r, eta, T(-1), st == 1 ? r0 : r, T(1), s);  // r -= A d
         const double rn = 1.0 / (2.0 * ch.sigma - rho);
         launch_bj_apply<T>(N, int(ne), r, dd, y, emap.as<int>(), cls_inv.template as<T>(),
                            cls_sym.as<int>(), uniq_inv.template as<T>(),
@@ -865,7 +870,7 @@ void Multigrid<T>::vcycle_on(const T* b, T* y, cudaStream_t s) {
     if (P->desc.coarse == SIP_COARSE_Q0) {
         // coarse correction on the element-wise constants: the residual's
         // (0,0) modes are the finest vertex-grid level's right-hand side
-        launch_apply_sip<T>(N, P->geom, y, pr.template as<T>(), eta_of<T>(P), T(-1), b, T(1), s);
+        launch_apply_sip<T>(N, P->op(), y, pr.template as<T>(), eta_of<T>(P), T(-1), b, T(1), s);
         launch_p_restrict<T>(ne, N, pr.template as<T>(), h[0].b.template as<T>(), s, 1);
         hcycle(0, s);
         launch_p_prolong_add<T>(ne, N, h[0].x.template as<T>(), y, s, 1);
@@ -874,7 +879,7 @@ void Multigrid<T>::vcycle_on(const T* b, T* y, cudaStream_t s) {
     }
     // r1 = R (b - A y)
     if (!residual_restrict(y, b, r1.template as<T>(), s)) {
-        launch_apply_sip<T>(N, P->geom, y, pr.template as<T>(), eta_of<T>(P), T(-1), b, T(1), s);
+        launch_apply_sip<T>(N, P->op(), y, pr.template as<T>(), eta_of<T>(P), T(-1), b, T(1), s);
         launch_p_restrict<T>(ne, N, pr.template as<T>(), r1.template as<T>(), s);
     }
     if (h.empty()) {
@@ -928,7 +933,7 @@ int Multigrid<T>::inner_pcg(const T* t, T* y, double rtol, int maxit, cudaStream
     launch_axpby<T>(n_u, T(1), z, T(0), dd, s);
     int it = 0;
     for (it = 1; it <= maxit; ++it) {
-        launch_apply_sip<T>(N, P->geom, dd, q, eta, T(1), nullptr, T(0), s);
+        launch_apply_sip<T>(N, P->op(), dd, q, eta, T(1), nullptr, T(0), s);
         launch_dot<T>(n_u, dd, q, scd + 1, wsd, s);
         launch_pcg_update<T>(n_u, dd, q, y, r, scd + 0, scd + 1, s);
         launch_dot<T>(n_u, r, r, scd + 2, wsd, s);
@@ -983,7 +988,7 @@ int inner_pcg_mixed(sip_problem* P, Workspace& W, const double* t, double* y, do
     launch_axpby<double>(n_u, 1.0, z, 0.0, dd, s);
     int it = 0;
     for (it = 1; it <= maxit; ++it) {
-        launch_apply_sip<double>(P->n, P->geom, dd, q, eta, 1.0, nullptr, 0.0, s);
+        launch_apply_sip<double>(P->n, P->op(), dd, q, eta, 1.0, nullptr, 0.0, s);
         launch_dot<double>(n_u, dd, q, scd + 1, wsd, s);
         launch_pcg_update<double>(n_u, dd, q, y, r, scd + 0, scd + 1, s);
         launch_dot<double>(n_u, r, r, scd + 2, wsd, s);
@@ -1024,6 +1029,11 @@ sip_status run_solve(sip_problem* P, const double* f_u, const double* g_p, doubl
     const double setup0 = P->setup_ms;
     P->ensure_setup(s);
     const double setup_ms = P->setup_ms - setup0;
+    struct StokesScope {
+        sip_problem* P;
+        ~StokesScope() { P->in_stokes = false; }
+    } scope{P};
+    P->in_stokes = P->stiff;
     const bool f32_inner = P->desc.precision == SIP_PREC_MIXED_F32_INNER;
     const bool mixed = P->desc.precision == SIP_PREC_MIXED || f32_inner;
     const size_t n_u = size_t(P->n_u), n_p = size_t(P->n_p), n = n_u + n_p;
@@ -1086,17 +1096,14 @@ sip_status run_solve(sip_problem* P, const double* f_u, const double* g_p, doubl
     auto project = [&](double* v) {
         if (singular) launch_zero_mean_pressure(size_t(P->ne), P->mp, v + n_u, wsd, s);
     };
-    // y = K v  (w_u = A v_u + B v_p, w_p = B^T v_u).  One application per outer
-    // iteration (25 of 1600 operator applies of the 128^2, k = 3 box solve): it
-    // stays in FP64 arithmetic, whose rounding sets the attainable residual the
-    // stopping tests were chosen on; with the more accurate fixed-point apply some
-    // solves stop one or two iterations earlier at the same tolerance.
-    OpGeom gK = P->geom;
-    if (gK.variant[0] == APPLY_AUTO || gK.variant[0] == APPLY_STAGE) gK.variant[0] = APPLY_ELEM2;
+    // y = K v  (w_u = A v_u + B v_p, w_p = B^T v_u), one application per outer
+    // iteration: FP64 arithmetic at every contrast
+    OpGeom gK = P->op();
+    if (!gK.fp64 && (gK.variant[0] == APPLY_AUTO || gK.variant[0] == APPLY_STAGE)) gK.variant[0] = APPLY_ELEM2;
     auto applyK = [&](const double* v, double* y) {
-        launch_apply_B<double>(P->k, P->geom, v + n_u, W.tu.as<double>(), s);
+        launch_apply_B<double>(P->k, P->op(), v + n_u, W.tu.as<double>(), s);
         launch_apply_sip<double>(P->n, gK, v, y, eta, 1.0, W.tu.as<double>(), 1.0, s);
-        launch_apply_Bt<double>(P->k, P->geom, v, y + n_u, s);
+        launch_apply_Bt<double>(P->k, P->op(), v, y + n_u, s);
     };
     int inner_total = 0, inner_max = 0, inner_calls = 0;
     // the inner PCG runs as one graph launch with a device-side loop unless
@@ -1110,7 +1117,7 @@ sip_status run_solve(sip_problem* P, const double* f_u, const double* g_p, doubl
     auto precond = [&](const double* v, double* z) {
         launch_vmul<double>(n_p, v + n_u, W.sinv.as<double>(), z + n_u, s);   // y_p = -S*^{-1} v_p
         project(z);
-        launch_apply_B<double>(P->k, P->geom, z + n_u, W.tu.as<double>(), s);
+        launch_apply_B<double>(P->k, P->op(), z + n_u, W.tu.as<double>(), s);
         launch_axpby<double>(n_u, 1.0, v, -1.0, W.tu.as<double>(), s);        // t = v_u - B y_p
         int its;
         if (f32_inner) {
@@ -1559,6 +1566,21 @@ __global__ void k_derive_eta(size_t n, const double* eta, float* ef, double* inv
     inv[g] = 1.0 / e;
     invf[g] = float(1.0 / e);
 }
+
+// positive doubles order as their bits
+__global__ void k_eta_range(size_t n, const double* eta, unsigned long long* range) {
+    sip::grid_dep_wait();
+    unsigned long long lo = ~0ull, hi = 0;
+    for (size_t g = size_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += size_t(gridDim.x) * blockDim.x) {
+        const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(eta[g]));
+        lo = b < lo ? b : lo;
+        hi = b > hi ? b : hi;
+    }
+    if (hi > 0) {
+        atomicMin(range, lo);
+        atomicMax(range + 1, hi);
+    }
+}
 }  // namespace
 
 void sip_problem::derive_eta(cudaStream_t s) {
@@ -1571,11 +1593,29 @@ void sip_problem::derive_eta(cudaStream_t s) {
     SIP_CHECK_LAUNCH();
 }
 
+void sip_problem::find_contrast(cudaStream_t s) {
+    if (contrast_known) return;
+    eta_range.alloc(2 * sizeof(double));
+    SIP_CUDA(cudaMemsetAsync(eta_range.ptr, 0xff, sizeof(double), s));
+    SIP_CUDA(cudaMemsetAsync(eta_range.as<double>() + 1, 0, sizeof(double), s));
+    sip::launch_k(k_eta_range, 64, 256, 0, s, size_t(ne), eta_d.as<double>(),
+                  eta_range.as<unsigned long long>());
+    SIP_CHECK_LAUNCH();
+    double r[2];
+    SIP_CUDA(cudaMemcpyAsync(r, eta_range.ptr, sizeof(r), cudaMemcpyDeviceToHost, s));
+    SIP_CUDA(cudaStreamSynchronize(s));
+    stiff = r[1] / r[0] > kFixedContrast;
+    contrast_known = true;
+}
+
 void sip_problem::ensure_setup(cudaStream_t s) {
     const double t0 = sip::now_ms();
     bool did = false;
     const bool fresh = (mg32 == nullptr || !mg32->ready) && (mg64 == nullptr || !mg64->ready);
-    if (fresh) sip::tune_apply(this, s);
+    if (fresh) {
+        find_contrast(s);
+        sip::tune_apply(this, s);
+    }
     if (desc.precision == SIP_PREC_MIXED || desc.precision == SIP_PREC_MIXED_F32_INNER) {
         if (!mg32) {
             mg32 = std::make_unique<sip::Multigrid<float>>();

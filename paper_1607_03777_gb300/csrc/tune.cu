@@ -87,14 +87,9 @@ double time_ms(F&& f, cudaStream_t s, int reps) {
 }
 
 template <typename T>
-void tune_apply_t(sip_problem* P, cudaStream_t s) {
+void tune_apply_t(sip_problem* P, OpGeom& g, cudaStream_t s) {
     const int t = sizeof(T) == 4 ? 1 : 0;
-    if (P->pin_apply[t] > 0) {   // pinned: code 5 = staged with 4 tile rows
-        P->geom.variant[t] = P->pin_apply[t] == 5 ? int(APPLY_STAGE) : P->pin_apply[t];
-        P->geom.stage_rows[t] = P->pin_apply[t] == 5 ? 4 : 2;
-        return;
-    }
-    const Key key{0, P->n, int(sizeof(T)), P->desc.nx, P->desc.ny};
+    const Key key{g.fp64 ? 2 : 0, P->n, int(sizeof(T)), P->desc.nx, P->desc.ny};
     int best = APPLY_AUTO;   // variant + 16 x stage rows
     if (!cached(key, best)) {
         const size_t n_u = size_t(P->n_u);
@@ -105,16 +100,16 @@ void tune_apply_t(sip_problem* P, cudaStream_t s) {
         const T* eta = eta_vec<T>(P);
         double tbest = 1e300;
         const int64_t launches = launch_counter();
-        const int saved_rows = P->geom.stage_rows[t];
+        const int saved_rows = g.stage_rows[t];
         for (int cand : {int(APPLY_ELEM2), int(APPLY_ELEM1), int(APPLY_TILE),
                          int(APPLY_STAGE) + 16 * 2, int(APPLY_STAGE) + 16 * 4,
                          sizeof(T) == 4 ? int(APPLY_WARP) : -1}) {
             if (cand < 0) continue;
-            P->geom.variant[t] = cand % 16;
-            P->geom.stage_rows[t] = cand / 16 ? cand / 16 : saved_rows;
+            g.variant[t] = cand % 16;
+            g.stage_rows[t] = cand / 16 ? cand / 16 : saved_rows;
             const double ms = time_ms(
                 [&] {
-                    launch_apply_sip<T>(P->n, P->geom, x.as<T>(), y.as<T>(), eta, T(1), nullptr,
+                    launch_apply_sip<T>(P->n, g, x.as<T>(), y.as<T>(), eta, T(1), nullptr,
                                         T(0), s);
                 },
                 s, 5);
@@ -123,39 +118,43 @@ void tune_apply_t(sip_problem* P, cudaStream_t s) {
                 best = cand;
             }
         }
-        P->geom.stage_rows[t] = saved_rows;
+        g.stage_rows[t] = saved_rows;
         launch_counter() = launches;
         store(key, best);
     }
-    P->geom.variant[t] = best % 16;
-    if (best / 16) P->geom.stage_rows[t] = best / 16;
+    g.variant[t] = best % 16;
+    if (best / 16) g.stage_rows[t] = best / 16;
 }
 
 }  // namespace
 
 void tune_apply(sip_problem* P, cudaStream_t s) {
-    if (P->n > 6) return;   // one kernel exists above degree 5
-    if (!autotune_on()) {
-        for (int t = 0; t < 2; ++t)
-            if (P->pin_apply[t] > 0) {
-                P->geom.variant[t] = P->pin_apply[t] == 5 ? int(APPLY_STAGE) : P->pin_apply[t];
-                P->geom.stage_rows[t] = P->pin_apply[t] == 5 ? 4 : 2;
-            }
-        return;
-    }
-    tune_apply_t<double>(P, s);
-    if (P->desc.precision != SIP_PREC_FP64) tune_apply_t<float>(P, s);
+    for (int t = 0; t < 2; ++t)
+        if (P->pin_apply[t] > 0) {   // pinned: code 5 = staged with 4 tile rows
+            P->geom.variant[t] = P->pin_apply[t] == 5 ? int(APPLY_STAGE) : P->pin_apply[t];
+            P->geom.stage_rows[t] = P->pin_apply[t] == 5 ? 4 : 2;
+        }
+    // one kernel exists above degree 5
+    const bool on = autotune_on() && P->n <= 6;
+    if (on && P->pin_apply[0] == 0) tune_apply_t<double>(P, P->geom, s);
+    if (on && P->pin_apply[1] == 0 && P->desc.precision != SIP_PREC_FP64) tune_apply_t<float>(P, P->geom, s);
+    P->geom_solve = P->geom;
+    P->geom_solve.fp64 = 1;
+    if (!P->stiff || P->pin_apply[0] > 0) return;
+    P->geom_solve.variant[0] = APPLY_AUTO;
+    P->geom_solve.stage_rows[0] = 2;
+    if (on) tune_apply_t<double>(P, P->geom_solve, s);
 }
 
 template <typename T>
-void Multigrid<T>::tune_smoother(cudaStream_t s) {
+void Multigrid<T>::tune_smoother(OpGeom& g, cudaStream_t s) {
     const int t = sizeof(T) == 4 ? 1 : 0;
     if (P->pin_fused[t] >= 0) {
-        P->geom.fused[t] = P->pin_fused[t];
+        g.fused[t] = P->pin_fused[t];
         return;
     }
     if (!autotune_on() || !cheb_elem_available(N) || !pd2.ptr) return;
-    const Key key{1, N, int(sizeof(T)), P->desc.nx, P->desc.ny};
+    const Key key{g.fp64 ? 3 : 1, N, int(sizeof(T)), P->desc.nx, P->desc.ny};
     int fused = 1;
     if (!cached(key, fused)) {
         T* b = pb.template as<T>();
@@ -173,13 +172,13 @@ void Multigrid<T>::tune_smoother(cudaStream_t s) {
         const int64_t launches = launch_counter();
         const double t_fused = time_ms(
             [&] {
-                launch_cheb_elem<T>(N, P->geom, d, r, r, eta, em, ci, csym, ui, einv, d, d2, y,
+                launch_cheb_elem<T>(N, g, d, r, r, eta, em, ci, csym, ui, einv, d, d2, y,
                                     T(0.5), T(0.5), false, s);
             },
             s, 5);
         const double t_split = time_ms(
             [&] {
-                launch_apply_sip<T>(N, P->geom, d, r, eta, T(-1), r, T(1), s);
+                launch_apply_sip<T>(N, g, d, r, eta, T(-1), r, T(1), s);
                 launch_bj_apply<T>(N, int(ne), r, d2, y, em, ci, csym, ui, einv, T(0.5), T(0.5),
                                    false, s);
             },
@@ -188,7 +187,16 @@ void Multigrid<T>::tune_smoother(cudaStream_t s) {
         fused = t_fused <= t_split ? 1 : 0;
         store(key, fused);
     }
-    P->geom.fused[t] = fused;
+    g.fused[t] = fused;
+}
+
+template <typename T>
+void Multigrid<T>::tune_smoother(cudaStream_t s) {
+    tune_smoother(P->geom, s);
+    if (sizeof(T) == 8 && P->stiff)
+        tune_smoother(P->geom_solve, s);
+    else
+        for (int t = 0; t < 2; ++t) P->geom_solve.fused[t] = P->geom.fused[t];
 }
 
 template void Multigrid<double>::tune_smoother(cudaStream_t);
