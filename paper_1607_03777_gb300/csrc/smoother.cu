@@ -246,6 +246,117 @@ __global__ void __launch_bounds__(256) k_bj_apply(const BJBatchArgs<T> a) {
     bj_body<N, T>(blockIdx.x * EB, a);
 }
 
+// CTAs per SM of k_bj_stream: what the kept row and two groups' operands leave
+template <int N, typename T>
+constexpr int bj_ctas() {
+    return sizeof(T) == 8 ? 3 : (N <= 4 ? 5 : (N == 5 ? 4 : 3));
+}
+
+// The same for one element set, a thread keeping its (element slot, row) over many
+// groups of EB elements.  Nearly all elements share the inverse of the interior class,
+// of which a row has N^2 / 2 entries of its parity: they stay in registers, and with
+// strides of two the residual's entries lie at fixed offsets from two per-thread bases,
+// so a product is one shared load and one FMA (bj_body spends two loads and the index
+// arithmetic of its parity loop on it).  The next group's operands are loaded while one
+// is computed.  Same order of summation as bj_body: same bits.  Elements of other
+// classes and unique blocks take its loops.
+template <int N, typename T>
+__global__ void __launch_bounds__(256, (bj_ctas<N, T>()))
+    k_bj_stream(const BJBatchArgs<T> a, int groups) {
+    grid_dep_wait();
+    constexpr int NN = N * N, NB = 2 * NN, H = (N + 1) / 2;
+    constexpr int EB = (256 / NB) > 0 ? (256 / NB) : 1;
+    __shared__ T sr[2][EB * NB];
+    const int q = threadIdx.x, el = q / NB, row = q % NB;
+    const size_t total = size_t(a.ne) * NB;
+    // the row's parity group: entries c NN + (j0 + 2 b) N + i0 + 2 a
+    const int cr = row / NN, jr = (row / N) % N, ir = row % N;
+    int base[2];
+    bool vi[2], vj[2];   // the last a, b lie inside the element
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int i0 = ((ir + (cr == 0 ? 1 : 0)) & 1) ^ (c == 0 ? 1 : 0);
+        const int j0 = ((jr + (cr == 1 ? 1 : 0)) & 1) ^ (c == 1 ? 1 : 0);
+        base[c] = c * NN + j0 * N + i0;
+        vi[c] = i0 + 2 * (H - 1) < N;
+        vj[c] = j0 + 2 * (H - 1) < N;
+    }
+    const bool keep = a.cls_sym && a.cls_sym[0] == 3;   // interior class, both symmetries
+    T m[2][H][H];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int b = 0; b < H; ++b)
+#pragma unroll
+            for (int i = 0; i < H; ++i)
+                m[c][b][i] = keep && (i < H - 1 || vi[c]) && (b < H - 1 || vj[c])
+                                 ? a.cls_inv[size_t(base[c] + 2 * b * N + 2 * i) * NB + row]
+                                 : T(0);
+    const T c1 = a.c1, c2 = a.c2;
+    const bool use_old = c1 != T(0), use_x = a.x && !a.x_zero;
+    struct In {
+        T r, old, x, scale;
+        int map;
+        bool act;
+    };
+    const auto load = [&](int g) {
+        In v{T(0), T(0), T(0), T(1), -1, false};
+        const size_t o = size_t(g) * (EB * NB) + q;
+        if (g >= groups || q >= EB * NB || o >= total) return v;
+        v.act = true;
+        v.r = a.r[o];
+        const int e = g * EB + el;
+        v.map = a.emap[e];
+        v.scale = a.eta_inv[e];
+        if (use_old) v.old = a.out[o];
+        if (use_x) v.x = a.x[o];
+        return v;
+    };
+    In cur = load(int(blockIdx.x));
+    int buf = 0;
+    for (int g = blockIdx.x; g < groups; g += gridDim.x) {
+        if (cur.act) sr[buf][q] = cur.r;
+        __syncthreads();
+        const In next = load(g + int(gridDim.x));
+        if (cur.act) {
+            const T* rr = sr[buf] + el * NB;
+            T acc = T(0), scale = cur.scale;
+            if (cur.map == -1 && keep) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int b = 0; b < H; ++b)
+#pragma unroll
+                        for (int i = 0; i < H; ++i)
+                            if ((N % 2 == 0 || i < H - 1 || vi[c]) && (N % 2 == 0 || b < H - 1 || vj[c]))
+                                acc += m[c][b][i] * rr[base[c] + 2 * b * N + 2 * i];
+            } else if (cur.map < 0) {
+                acc = block_row_apply<N, T>(a.cls_inv + size_t(-cur.map - 1) * NB * NB, rr, row,
+                                            a.cls_sym ? a.cls_sym[-cur.map - 1] : 0);
+            } else {
+                scale = T(1);
+                const size_t off = size_t(cur.map) * NB * NB;
+                if (sizeof(T) == 4 && a.uniq_hi && a.uniq_hi[cur.map] && a.uniq_inv64) {
+                    const double* M = a.uniq_inv64 + off;
+                    double a64 = 0.0;
+#pragma unroll 8
+                    for (int q2 = 0; q2 < NB; ++q2) a64 += M[q2 * NB + row] * double(rr[q2]);
+                    acc = T(a64);
+                } else {
+                    acc = block_row_apply<N, T>(a.uniq_inv + off, rr, row, 0);
+                }
+            }
+            T v = c2 * scale * acc;
+            if (use_old) v += c1 * cur.old;
+            const size_t o = size_t(g) * (EB * NB) + q;
+            a.out[o] = v;
+            if (a.x) a.x[o] = a.x_zero ? v : cur.x + v;
+        }
+        cur = next;
+        buf ^= 1;
+    }
+}
+
 // Many block-Jacobi applies in one launch: CTA b serves member items[b].x
 // (arguments args[items[b].x]), element group items[b].y; members with
 // active[m] == 0 are skipped.
@@ -298,6 +409,19 @@ void bj_apply_n(int ne, const T* r, T* out, T* x, const int* emap, const T* cls_
     const int blocks = (ne + EB - 1) / EB;
     const BJBatchArgs<T> a{ne, r, out, x, emap, cls_inv, cls_sym, uniq_inv, eta, uniq_hi,
                            uniq_inv64, c1, c2, x_zero ? 1 : 0};
+    // The row kept in registers pays once every CTA serves more than three groups:
+    // FP32 V-cycle 256^2, k = 4: 334 -> 272 us, 192^2, k = 2: 113 -> 106 us, but 64^2,
+    // k = 5 (3.0 groups): 99 -> 105 us.  In FP64 it pays for short rows (256^2, k = 2:
+    // 42.4 -> 33.9 us an apply); above k = 2 the FP64 pipe bounds both kernels and more
+    // CTAs per SM win (k = 4: 141.6 against 146.8 us).
+    if constexpr (sizeof(T) == 4 || N <= 3) {
+        const int resident = 152 * bj_ctas<N, T>();
+        if (blocks > 3 * resident) {
+            launch_k(k_bj_stream<N, T>, unsigned(resident), 256, 0, s, a, blocks);
+            SIP_CHECK_LAUNCH();
+            return;
+        }
+    }
     launch_k(k_bj_apply<N, T>, blocks, 256, 0, s, a);
     SIP_CHECK_LAUNCH();
 }
