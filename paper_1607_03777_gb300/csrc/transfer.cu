@@ -57,7 +57,21 @@ __global__ void k_pcd(int nx, int ny, const T* __restrict__ v, T* __restrict__ o
     out[g] = T(acc);
 }
 
-// The same added to the Q^2_1 modes of a degree N - 1 vector.
+// Exact FP64 value of an FP32 number by integer operations: the conversion
+// instruction runs on the FP64 pipe (under 2 lanes per clock and SM), which bounds
+// the transfers of the FP32 cycle.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m >= 0x7f800000u || (m < 0x00800000u && m != 0)) return double(v);   // inf, NaN, subnormal
+    const unsigned hi = m == 0 ? b : (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
+    return __hiloint2double(int(hi), m == 0 ? 0 : int(b << 29));
+}
+
+// P P_cd v added to the Q^2_1 modes of a degree N - 1 vector, one thread per mode.
+// The weights hatw(i, p) hatw(j, q) of a thread differ in sign only; FP32 data is
+// widened by integer operations (5 FP64 operations per mode instead of 13; with it and the
+// same in k_rdc a FP32 V-cycle of 256^2, k = 2: 178 -> 172 us).
 template <typename T>
 __global__ void k_pcd_add(int nx, int ny, int N, const T* __restrict__ v, T* __restrict__ y) {
     grid_dep_wait();
@@ -67,10 +81,16 @@ __global__ void k_pcd_add(int nx, int ny, int N, const T* __restrict__ v, T* __r
     const size_t e = g / 8;
     const int l = int(g % 8), c = l / 4, j = (l / 2) % 2, i = l % 2;
     const int ex = int(e % nx), ey = int(e / nx);
+    const double w = i + j == 0 ? kInvSqrt2 * kInvSqrt2
+                                : (i + j == 1 ? kInvSqrt2 * kInvSqrt6 : kInvSqrt6 * kInvSqrt6);
     double acc = 0.0;
+#pragma unroll
     for (int q = 0; q < 2; ++q)
-        for (int p = 0; p < 2; ++p)
-            acc += hatw(i, p) * hatw(j, q) * double(v[2 * (size_t(ey + q) * (nx + 1) + ex + p) + c]);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const bool minus = (i == 1 && p == 0) != (j == 1 && q == 0);
+            acc += (minus ? -w : w) * widen(v[2 * (size_t(ey + q) * (nx + 1) + ex + p) + c]);
+        }
     y[e * 2 * N * N + c * N * N + j * N + i] += T(acc);
 }
 
@@ -84,15 +104,19 @@ __global__ void k_rdc(int nx, int ny, const T* __restrict__ r, T* __restrict__ o
     const size_t v = g / 2;
     const int vx = int(v % (nx + 1)), vy = int(v / (nx + 1));
     double acc = 0.0;
+#pragma unroll
     for (int q = 0; q < 2; ++q) {          // vertex is corner q (in y) of element row vy - q
         const int ey = vy - q;
         if (ey < 0 || ey >= ny) continue;
+#pragma unroll
         for (int p = 0; p < 2; ++p) {
             const int ex = vx - p;
             if (ex < 0 || ex >= nx) continue;
             const T* re = r + (size_t(ey) * nx + ex) * 8 + c * 4;
+#pragma unroll
             for (int j = 0; j < 2; ++j)
-                for (int i = 0; i < 2; ++i) acc += hatw(i, p) * hatw(j, q) * double(re[j * 2 + i]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) acc += hatw(i, p) * hatw(j, q) * widen(re[j * 2 + i]);
         }
     }
     out[g] = T(acc);
