@@ -328,13 +328,15 @@ struct sip_problem {
     sip::OpGeom geom{};      // the SIP operator of degree k
     // Schedule of a Stokes solve whose viscosity contrast is above kFixedContrast:
     // FP64 arithmetic in every operator.  There the saddle system's attainable
-    // residual in FP64 comes near the tolerances in use (3e-9 of ||b|| for a stiff
-    // box of contrast 1e4 at 128^2, k = 3); a solve whose true residual misses the
-    // tolerance when its recurrence meets it continues from rounding errors, and the
-    // solution then depends on the operators' last bits by 1e-9 to 5e-7 of its norm.
-    // Below, two roundings of the operators agree to 1e-11 after a solve (40 x 32 to
-    // 80 x 64, k = 2 to 4, contrast 19 to 170).  128^2, k = 3, contrast 1e4: 137 ms a step,
-    // 101 ms with the fixed-point operator.
+    // residual in FP64 comes near the tolerances in use; a solve whose true residual
+    // misses the tolerance when its recurrence meets it continues from rounding
+    // errors, and the solution then depends on the operators' last bits: two equally
+    // accurate operators gave velocities 1e-9 to 4e-8 of their norm apart in 2 of 12
+    // solves (128^2, k = 3, contrast 1e4; rtol 1e-8), once 5e-7 (64^2, k = 2, 300).
+    // Below, they agreed to 1e-12 after a solve (25 solves of 40 x 32 to 80 x 64
+    // elements, k = 2 to 4, contrast 19 to 170) and to 4e-11 in 96 batched ones
+    // (32^2, contrast 100).  128^2, k = 3, contrast 1e4: 137 ms a step, 101 ms with the
+    // fixed-point operator.
     sip::OpGeom geom_solve{};
     static constexpr double kFixedContrast = 128.0;
     sip::DeviceBuffer eta_range;   // bits of the smallest and largest viscosity
