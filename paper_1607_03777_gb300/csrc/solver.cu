@@ -895,6 +895,11 @@ void Multigrid<T>::vcycle_on(const T* b, T* y, cudaStream_t s) {
 
 template <typename T>
 void Multigrid<T>::vcycle(const T* r, T* z, cudaStream_t s) {
+    // the graph holds the other schedule's kernels (FP32: the same in both)
+    if (sizeof(T) == 8 && P->in_stokes && r != z) {
+        vcycle_on(r, z, s);
+        return;
+    }
     if (r != vin.template as<T>())
         SIP_CUDA(cudaMemcpyAsync(vin.ptr, r, n_u * sizeof(T), cudaMemcpyDeviceToDevice, s));
     SIP_CUDA(cudaGraphLaunch(graph, s));
