@@ -114,9 +114,20 @@ __device__ __forceinline__ bool fix_load(const FixArgs<TS>& a, const fix::Mesh& 
         seta[s] = v;
     }
     const int grp = (threadIdx.x / 32) * EPW + (threadIdx.x % 32) / SEG, ls = threadIdx.x % SEG;
+    // this lane's entries: conversion factor, component, whether it is a constant mode,
+    // and the bits of its magnitude that count for either component's exponent
     double ss[CH];
+    bool second[CH], mean[CH];
+    unsigned of0[CH], of1[CH];
 #pragma unroll
-    for (int c = 0; c < CH; ++c) ss[c] = a.ss[(ls + c * SEG) % L::NN];
+    for (int c = 0; c < CH; ++c) {
+        const int q = ls + c * SEG;
+        ss[c] = a.ss[q % L::NN];
+        second[c] = q >= L::NN;
+        mean[c] = q == 0 || q == L::NN;
+        of0[c] = mean[c] || second[c] ? 0u : 0x7fffffffu;
+        of1[c] = mean[c] || !second[c] ? 0u : 0x7fffffffu;
+    }
     // every lane of a warp takes the same number of rounds (shuffles below)
     constexpr int ROUNDS = (L::NS + STEP * U - 1) / (STEP * U);
 #pragma unroll 1
@@ -138,39 +149,40 @@ __device__ __forceinline__ bool fix_load(const FixArgs<TS>& a, const fix::Mesh& 
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             const int s = (r * U + t) * STEP + grp;
-            unsigned m = 0;
+            // largest magnitude (high words) of each component but its constant mode
+            unsigned m0 = 0, m1 = 0;
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
-                const unsigned h = unsigned(__double2hiint(v[t][c])) & 0x7fffffffu;
-                m = h > m ? h : m;
+                const unsigned h = unsigned(__double2hiint(v[t][c]));
+                m0 = max(m0, h & of0[c]);
+                m1 = max(m1, h & of1[c]);
             }
             if constexpr (SEG == 32) {
-                m = __reduce_max_sync(0xffffffffu, m);
+                m0 = __reduce_max_sync(0xffffffffu, m0);
+                m1 = __reduce_max_sync(0xffffffffu, m1);
             } else {
 #pragma unroll
                 for (int o = SEG / 2; o > 0; o >>= 1) {
-                    const unsigned n = __shfl_xor_sync(0xffffffffu, m, o);
-                    m = n > m ? n : m;
+                    m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+                    m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
                 }
             }
-            const int e = int(m >> 20);
-            bool fits = e >= fix::E_MIN && e <= fix::E_MAX;
-            if (e == 0) {   // all zero (or subnormal)
+            const int e0 = int(m0 >> 20), e1 = int(m1 >> 20);
+            int* above = reinterpret_cast<int*>(su + s * L::XS + L::NB);   // fix::mean_pack
 #pragma unroll
-                for (int c = 0; c < CH; ++c) bad = bad || v[t][c] != 0.0;
-            } else {
-                bad = bad || !fits;
-            }
-            if (s < L::NS) {
-#pragma unroll
-                for (int c = 0; c < CH; ++c) {
-                    const int q = ls + c * SEG;
-                    if (q < L::NB)
-                        su[s * L::XS + q] =
-                            fits ? fix::to_int(v[t][c] * fix::in_factor<N>(ss[c], e)) : 0;
+            for (int c = 0; c < CH; ++c) {
+                const int q = ls + c * SEG;
+                const unsigned h = unsigned(__double2hiint(v[t][c])) & 0x7fffffffu;
+                const int ec = second[c] ? e1 : e0, e = mean[c] ? int(h >> 20) : ec;   // grid of this entry
+                const bool fits = e >= fix::E_MIN && e <= fix::E_MAX;
+                // outside the range, unless zero
+                bad = bad || (!fits && (h | unsigned(__double2loint(v[t][c]))) != 0);
+                if (s < L::NS && q < L::NB) {
+                    su[s * L::XS + q] = fits ? fix::to_int(v[t][c] * fix::in_factor<N>(ss[c], e)) : 0;
+                    if (mean[c]) above[second[c] ? 1 : 0] = e - ec;
                 }
-                if (ls == 0) se[s] = e;
             }
+            if (s < L::NS && ls == 0) se[s] = fix::expo_pack(e0, e1);
         }
     }
     return bad;
@@ -252,7 +264,7 @@ constexpr int min_blocks() {
     using L = fix::Tile<N, TW, TH>;
     const int fit = int((228 * 1024) / (L::BYTES + 1024)), reg = 65536 / (L::NT * 96);
     const int b = fit < reg ? fit : reg;
-    return b > 1 ? b : 1;
+    return b > 4 ? 4 : (b > 1 ? b : 1);   // more CTAs only serve meshes too small to fill them
 }
 
 template <int N, int TW, int TH, typename TS>

@@ -11,18 +11,27 @@
 // high products (three wide multiply-adds): the viscosities, the
 // geometric / mass factors (hy/hx) 2/(2b+1), and the penalty.
 //
-// Scaling.  Element K's coefficients become integers U = s_i s_j u 2^FRAC /
-// 2^e_K, with 2^e_K just above max |u| on K and s_i = sqrt((2i+1)/2); FRAC is
-// the largest for which no sum that is multiplied can reach 2^63 (55 bits at
-// k = 5, 57 at k = 3): a finer grid than FP64's on the element's largest entry.
-// Sums over one element are exact; a jump is formed on the coarser grid of the
+// Scaling.  The coefficients of one component on element K become integers
+// U = s_i s_j u 2^FRAC / 2^e, with 2^e just above the largest |u| of that component's
+// modes but the constant one, and s_i = sqrt((2i+1)/2); FRAC is the largest for
+// which no sum that is multiplied can reach 2^63 (55 bits at k = 5, 57 at k = 3): a
+// finer grid than FP64's on the component's largest entry, and a coarser one than
+// FP64's on an entry more than 2^(FRAC - 53) below it.  The result's error is thus
+// bounded by 2^-53 of the largest term that the component brings into the element, not
+// of each entry's own terms.  The constant mode (0, 0) has an exponent of its own:
+// it enters the jumps of the lines m = 0 and the cross sums over them and nothing
+// else, and a translation of both sides of a face leaves nothing, whatever else moves
+// on top of it.  (With one exponent for all entries of an element, u_x = 1 and u_y of
+// size 1e-12 lost 38 of the 53 bits of what u_y gives, and a nearly rigid motion of a
+// stiff inclusion is such a field; the separate exponents cost 2 to 10 % of an apply.)
+// Sums over one component are exact; a jump is formed on the coarser grid of the
 // face's two elements, the same on both sides.  Viscosities are 62-bit
 // mantissas with exponents relative to the largest of K and its neighbours.
 // Products are rounded to a unit that each line picks from the magnitudes it
-// has, so a large factor (penalty, stiff neighbour) costs no resolution where
-// what it multiplies is small.  Rounding of traces thus cancels between the
-// elements of a face as it does in FP64, which matters: the coarse levels
-// amplify a net force on a floating stiff inclusion by 1e4 to 1e7.
+// has, so a large factor (penalty, stiff neighbour, the other component) costs no
+// resolution where what it multiplies is small or zero.  Rounding of traces thus
+// cancels between the elements of a face as it does in FP64, which matters: the
+// coarse levels amplify a net force on a floating stiff inclusion by 1e4 to 1e7.
 //
 // With kx_b = (hy/hx) 2/(2b+1), J = own - neighbour trace, d = reference normal
 // derivative trace, s = +-1 the side, the result modes along an x-line (row b)
@@ -35,8 +44,9 @@
 //           eta_K S_K + eta_N S_N, S = sum_{m>b, odd} v_n[m]   (tangential),
 // and y = s_a s_b W.  Boundary faces are ghosts: v_N = -v or +v, d_N likewise.
 //
-// Host and device: tests/test_fix_host.py compiles this file with the host
-// compiler and runs the same phases tile by tile against the oracle.
+// Host and device: tests/test_fix_host.py and tests/test_fix_parts.py compile this file
+// with the host compiler and run the same phases tile by tile against the oracle and the
+// operator in extended precision.
 #pragma once
 
 #include <cmath>
@@ -164,13 +174,24 @@ struct Shift {
 };
 FIX_HD Shift shift_by(int n) {
     Shift s;
-    s.l = n < 0 ? -n : 0;
+    s.l = n < 0 ? (n > -62 ? -n : 62) : 0;   // that far up: only zeros
     s.n = n < 0 ? 0 : (n < 62 ? n : 62);
     s.half = n < 59 ? (i64(1) << s.n) >> 1 : 0;   // at most 2^57: no overflow
     return s;
 }
 FIX_HD i64 shr(i64 x, Shift s) { return ((x << s.l) + s.half) >> s.n; }
-FIX_HD i64 align(i64 x, Shift s) { return (x + s.half) >> s.n; }   // n >= 0
+// the same for n >= 0 and |x| < 2^62
+struct Down {
+    int n;
+    i64 half;
+};
+FIX_HD Down down_by(int n) {
+    Down s;
+    s.n = n < 62 ? n : 62;
+    s.half = (i64(1) << s.n) >> 1;
+    return s;
+}
+FIX_HD i64 align(i64 x, Down s) { return (x + s.half) >> s.n; }
 FIX_HD i64 prod(i64 t, Wt w, Shift s) { return shr(mulhi(t, w), s); }
 
 // high word of |t| (bitwise complement for negative t), for magnitude bounds
@@ -186,6 +207,17 @@ FIX_HD int bit_length(unsigned v) {
 #endif
 }
 FIX_HD int imax(int a, int b) { return a > b ? a : b; }
+FIX_HD int imin(int a, int b) { return a < b ? a : b; }
+// bit_length(mag(t)), or for zero a number that no unit depends on
+constexpr int NONE = -16000;
+FIX_HD int length(i64 t) { return t == 0 ? NONE : bit_length(mag(t)); }
+FIX_HD int bit_length64(i64 t) {   // of |t|
+#ifdef __CUDA_ARCH__
+    return 64 - __clzll(t < 0 ? -t : t);
+#else
+    return t ? 64 - __builtin_clzll((unsigned long long)(t < 0 ? -t : t)) : 0;
+#endif
+}
 FIX_HD Wt weight(i64 eta, i64 k) { return split(mulhi(eta, split(k)) << 2); }
 
 FIX_HD i64 bits_of(double v) {
@@ -256,16 +288,25 @@ struct Tile {
     static constexpr int NN = N * N, NB = 2 * NN;
     static constexpr int NEL = TW * TH, NH = 2 * TW + 2 * TH, NS = NEL + NH;
     static constexpr int NT = NEL * N;              // one thread per (element, line)
-    // odd strides: lanes that walk elements or entries hit distinct banks
-    static constexpr int XS = NB + 1, EP = NEL + 1, HP = NH + 1;
+    // faces of the tile's elements: x-normals y (TW + 1) + x, then y-normals y TW + x
+    static constexpr int NFX = (TW + 1) * TH, NF = NFX + TW * (TH + 1);
+    // odd strides: lanes that walk entries of one element hit distinct banks
+    static constexpr int XS = NB + 1, EP = NEL + 1;
+    // entries of the elements; the constant modes on grids of their own, and in the
+    // word behind the entries how far their exponents lie above the component's
+    // (mean_pack)
     static constexpr int O_U = 0;                   // in 8-byte words
     static constexpr int O_T = O_U + NS * XS;       // traces [(F 2 + c) N + m][val, der][element]
-    static constexpr int O_H = O_T + 16 * N * EP;   // halo traces [c N + m][val, der][halo element]
-    static constexpr int O_W = O_H + 4 * N * HP;    // results [mode][element]
+    static constexpr int O_H = O_T + 16 * N * NEL;  // halo traces [c N + m][val, der][halo element]
+    static constexpr int O_W = O_H + 4 * N * NH;    // results [mode][element]
     static constexpr int O_C = O_W + NB * EP;       // cross terms [mode][element]
-    static constexpr int O_ETA = O_C + NB * EP;
-    static constexpr int O_E = O_ETA + NS;          // ints: e[NS], E[NEL], ref[NEL], row units[2 N][NEL]
-    static constexpr size_t BYTES = size_t(O_E) * 8 + size_t(NS + (2 + 2 * N) * NEL) * 4;
+    static constexpr int O_M = O_C + NB * NEL;      // constant modes' jumps [c][face]
+    static constexpr int O_ETA = O_M + 2 * NF;
+    // ints: e[NS] (expo_pack), surroundings[NEL] (expo_pack of E and E + ref), row units
+    // [2 N][NEL]; then exponents of the jumps [c][face] (short)
+    static constexpr int O_E = O_ETA + NS;
+    static constexpr int I_R = NS, I_U = NS + NEL, I_M = I_U + 2 * N * NEL;
+    static constexpr size_t BYTES = size_t(O_E) * 8 + size_t(I_M) * 4 + 2 * NF * 2;
     static_assert(NEL % 32 == 0, "a warp serves one line index");
 };
 
@@ -273,6 +314,13 @@ struct Mesh {
     int nx, ny, ex0, ey0;
     int bc[4];
 };
+
+// Biased exponents of an element's components in one int, and those of its constant
+// modes relative to them in one word.
+FIX_HD int expo_pack(int e0, int e1) { return e0 + (e1 - e0) * 65536; }
+FIX_HD int expo(int packed, int c) { return (packed & 0xffff) + (c ? packed >> 16 : 0); }
+FIX_HD i64 mean_pack(int d0, int d1) { return i64(unsigned(d0)) | (i64(d1) << 32); }
+FIX_HD int mean_above(i64 packed, int c) { return c ? int(packed >> 32) : int(packed); }
 
 // Staged element s of the tile: its mesh position; false outside the mesh.
 template <int N, int TW, int TH>
@@ -294,20 +342,22 @@ FIX_HD bool staged_at(const Mesh& g, int s, int& ex, int& ey) {
     return ex >= 0 && ex < g.nx && ey >= 0 && ey < g.ny;
 }
 
-// Staged index of the neighbour of tile element el across face F, from its
-// coordinates.  (Written as `F == 0 ? (x > 0 ? el - 1 : ...)` nvcc 13.0 returned
-// el - 2 on the device where F is a compile-time 0; the GPU tests compare this
-// file's results on both sides.)
+// Staged index of the element at (x, y) of the tile or its halo.
 template <int N, int TW, int TH>
-FIX_HD int staged_nbr(int el, int F) {
+FIX_HD int staged_index(int x, int y) {
     using L = Tile<N, TW, TH>;
-    const int x = el % TW + (F == 1 ? 1 : 0) - (F == 0 ? 1 : 0);
-    const int y = el / TW + (F == 3 ? 1 : 0) - (F == 2 ? 1 : 0);
     if (x < 0) return L::NEL + 2 * TW + y;
     if (x >= TW) return L::NEL + 2 * TW + TH + y;
     if (y < 0) return L::NEL + x;
     if (y >= TH) return L::NEL + TW + x;
     return y * TW + x;
+}
+
+// Staged index of the neighbour of tile element el across face F.
+template <int N, int TW, int TH>
+FIX_HD int staged_nbr(int el, int F) {
+    return staged_index<N, TW, TH>(el % TW + (F == 1 ? 1 : 0) - (F == 0 ? 1 : 0),
+                                   el / TW + (F == 3 ? 1 : 0) - (F == 2 ? 1 : 0));
 }
 
 FIX_HD bool has_nbr(const Mesh& g, int ex, int ey, int F) {
@@ -334,10 +384,51 @@ FIX_HD void ends(const i64 (&U)[N], i64 (&v)[2], i64 (&d)[2]) {
     d[1] = dn + de;
 }
 
+// Entries of line m but the constant mode.
 template <int N>
 FIX_HD void load_line(const i64* u, int dir, int m, i64 (&U)[N]) {
 #pragma unroll
     for (int i = 0; i < N; ++i) U[i] = dir == 0 ? u[m * N + i] : u[i * N + m];
+    if (m == 0) U[0] = 0;
+}
+
+// Jumps of the constant modes (whose value trace on the line m = 0 is the same at every
+// end) across face f of the tile, the element on the low side less the one on the high
+// side, per component on the finest grid that holds it, with that grid's exponent (NONE:
+// no jump).  A ghost has the opposite value, or the same where the boundary condition
+// leaves no jump.
+template <int N, int TW, int TH>
+FIX_HD void mean_jumps(const Mesh& g, const i64* su, const int* se, int f, i64* jump, short* expo_of) {
+    using L = Tile<N, TW, TH>;
+    constexpr int FRAC = Bound<N>::FRAC;
+    const bool xn = f < L::NFX;
+    const int r = xn ? f : f - L::NFX, w = xn ? TW + 1 : TW, x = r % w, y = r / w;
+    const int at = xn ? g.ex0 + x : g.ey0 + y, end = xn ? g.nx : g.ny;   // of the high element
+    const bool inside = at <= end && (xn ? g.ey0 + y < g.ny : g.ex0 + x < g.nx);
+    const int l = staged_index<N, TW, TH>(x - (xn ? 1 : 0), y - (xn ? 0 : 1)), h = staged_index<N, TW, TH>(x, y);
+    const i64 *u = su + l * L::XS, *v = su + h * L::XS;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        i64 d = 0;
+        int lo = NONE;
+        if (inside) {
+            const int a = expo(se[l], c) + mean_above(u[L::NB], c), b = expo(se[h], c) + mean_above(v[L::NB], c);
+            int e = imax(a, b);
+            if (at > 0 && at < end) {
+                d = align(u[c * L::NN], down_by(e - a)) - align(v[c * L::NN], down_by(e - b));
+            } else {
+                const int kind = g.bc[(xn ? 0 : 2) + (at > 0 ? 1 : 0)];
+                e = at > 0 ? a : b;
+                if (kind == 2 || (kind == 0 && c == (xn ? 0 : 1)))
+                    d = at > 0 ? u[c * L::NN] << 1 : -(v[c * L::NN] << 1);
+            }
+            const int up = imax(FRAC - bit_length64(d), 0);
+            if (d != 0) lo = e - up;
+            d <<= up;
+        }
+        jump[c * L::NF + f] = d;
+        expo_of[c * L::NF + f] = short(lo);
+    }
 }
 
 // Phase 1: traces of the tile's elements (all faces) and of the halo
@@ -352,19 +443,20 @@ FIX_HD void phase_traces(int tid, const Mesh& g, i64* sm) {
     if (tid < L::NEL) {
         int ex, ey, E = 0, R = -2000;
         if (staged_at<N, TW, TH>(g, el, ex, ey)) {
-            E = se[el];
+            E = imax(expo(se[el], 0), expo(se[el], 1));
             R = eta_exp(eta[el]);
             for (int F = 0; F < 4; ++F)
                 if (has_nbr(g, ex, ey, F)) {
                     const int n = staged_nbr<N, TW, TH>(el, F);
-                    E = se[n] > E ? se[n] : E;
+                    E = imax(E, imax(expo(se[n], 0), expo(se[n], 1)));
                     const int r = eta_exp(eta[n]);
                     R = r > R ? r : R;
                 }
         }
-        se[L::NS + el] = E;
-        se[L::NS + L::NEL + el] = R;
+        se[L::I_R + el] = expo_pack(E, E + R);
     }
+    for (int f = tid; f < L::NF; f += L::NT)
+        mean_jumps<N, TW, TH>(g, su, se, f, sm + L::O_M, reinterpret_cast<short*>(se + L::I_M));
 #pragma unroll
     for (int dir = 0; dir < 2; ++dir)
 #pragma unroll
@@ -374,9 +466,9 @@ FIX_HD void phase_traces(int tid, const Mesh& g, i64* sm) {
             ends<N>(U, v, d);
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
-                i64* t = st + (((2 * dir + s) * 2 + c) * N + m) * 2 * L::EP + el;
+                i64* t = st + (((2 * dir + s) * 2 + c) * N + m) * 2 * L::NEL + el;
                 t[0] = v[s];
-                t[L::EP] = d[s];
+                t[L::NEL] = d[s];
             }
         }
     for (int q = tid; q < L::NH * N; q += L::NT) {
@@ -387,9 +479,9 @@ FIX_HD void phase_traces(int tid, const Mesh& g, i64* sm) {
             i64 U[N], v[2], d[2];
             load_line<N>(su + (L::NEL + h) * L::XS + c * L::NN, F / 2, mm, U);
             ends<N>(U, v, d);
-            i64* t = sh + (c * N + mm) * 2 * L::HP + h;
+            i64* t = sh + (c * N + mm) * 2 * L::NH + h;
             t[0] = F & 1 ? v[1] : v[0];
-            t[L::HP] = F & 1 ? d[1] : d[0];
+            t[L::NH] = F & 1 ? d[1] : d[0];
         }
     }
 }
@@ -406,12 +498,13 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
     i64 *sw = sm + L::O_W, *sc = sm + L::O_C;
     const double* seta = reinterpret_cast<const double*>(sm + L::O_ETA);
     int* se = reinterpret_cast<int*>(sm + L::O_E);
-    int* unit = se + L::NS + 2 * L::NEL;
+    int* unit = se + L::I_U;
     const int el = tid % L::NEL, m = tid / L::NEL;
     int ex, ey;
     if (!staged_at<N, TW, TH>(g, el, ex, ey)) return;
-    const int E = se[L::NS + el], ref = se[L::NS + L::NEL + el];
-    const int oK = E - se[el];   // exponent offsets: own, neighbour, face
+    // E: the reference exponent (offsets below it may be negative); of each component
+    const int E = expo(se[L::I_R + el], 0), ref = se[L::I_R + el] >> 16, pK = se[el];
+    const int oK[2] = {E - expo(pK, 0), E - expo(pK, 1)};   // exponent offsets: own
     const double etaK = seta[el];
     const i64 mK = eta_mant(etaK);
     const int rK = ref - eta_exp(etaK);
@@ -419,35 +512,52 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
     const Wt wC = split(mK), wK = weight(mK, k.km[DIR][m]);
     // per side: neighbour traces (or a ghost's multiples), weights, exponents
     const i64 *op[2], *np[2];
-    int ns[2], oN[2], oF[2], rN[2], rP[2], kind[2];
-    Shift aK[2], aN[2];   // own and neighbour traces to the face's exponent
+    int ns[2], oN[2][2], rN[2], rP[2], kind[2];   // oN: offsets of the neighbour's components
+    // per side and component: the grid of the jumps (its offset), own and neighbour traces
+    // to it, the constant mode's jump.  Both sides of a face form a jump on one grid, so
+    // that what one element gains the other loses, to the last bit of the jump.
+    int oG[2][2];
+    Down aK[2][2], aN[2][2];
+    i64 mj[2][2];
     Wt wN[2], wP[2], wCN[2];
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
         const int F = 2 * DIR + s;
-        op[s] = st + F * 4 * N * L::EP + el;
+        op[s] = st + F * 4 * N * L::NEL + el;
         np[s] = op[s];
-        ns[s] = L::EP;
-        oN[s] = oK;
+        ns[s] = L::NEL;
         kind[s] = 1 + g.bc[F];
         double eN = etaK;
+        int pN = pK;
         if (has_nbr(g, ex, ey, F)) {
             const int n = staged_nbr<N, TW, TH>(el, F);
             kind[s] = 0;
             if (n < L::NEL) {
-                np[s] = st + (F ^ 1) * 4 * N * L::EP + n;
+                np[s] = st + (F ^ 1) * 4 * N * L::NEL + n;
             } else {
                 np[s] = sh + (n - L::NEL);
-                ns[s] = L::HP;
+                ns[s] = L::NH;
             }
-            oN[s] = E - se[n];
+            pN = se[n];
             eN = seta[n];
         }
-        // both sides of a face form its jump on one grid, so that what one element
-        // gains the other loses, to the last bit of the jump
-        oF[s] = oN[s] < oK ? oN[s] : oK;
-        aK[s] = shift_by(oK - oF[s]);
-        aN[s] = shift_by(oN[s] - oF[s]);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            oN[s][c] = E - expo(pN, c);
+            oG[s][c] = imin(oK[c], oN[s][c]);
+            mj[s][c] = 0;
+            // the constant modes are part of the jumps on line 0, and of the tangential
+            // component's in the normal one's cross sums on the odd lines
+            if (m == 0 || (c != DIR && m % 2 == 1)) {
+                const int f = c * L::NF + (DIR == 0 ? (el / TW) * (TW + 1) + el % TW + s : L::NFX + el + s * TW);
+                const int lo = reinterpret_cast<const short*>(se + L::I_M)[f];
+                oG[s][c] = imin(oG[s][c], E - lo);
+                const i64 j = align(sm[L::O_M + f], down_by(E - oG[s][c] - lo));
+                mj[s][c] = s ? j : -j;
+            }
+            aK[s][c] = down_by(oK[c] - oG[s][c]);
+            aN[s][c] = down_by(oN[s][c] - oG[s][c]);
+        }
         const i64 mN = eta_mant(eN);
         rN[s] = ref - eta_exp(eN);
         wN[s] = weight(mN, k.km[DIR][m]);
@@ -463,23 +573,28 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
         i64 U[N], v[2], d[2];
         load_line<N>(su + el * L::XS + c * L::NN, DIR, m, U);
         ends<N>(U, v, d);
-        // per side: jump, own and neighbour derivative, own and neighbour cross sums
+        // per side: jump, own and neighbour derivative, own and neighbour cross sums;
+        // offset of the own cross sums' grid
         i64 J[2], O[2], Dn[2], X[2], Xn[2];
+        int oX[2];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
-            i64 x = 0, xn = 0;
+            constexpr int tc = 1 - DIR;
+            i64 x = normal && m % 2 == 1 ? mj[s][tc] : 0, xn = 0;
+            const i64 jm = m == 0 ? mj[s][c] : 0;
+            oX[s] = normal ? oG[s][tc] : oK[DIR];
             if (kind[s] == 0) {
                 const i64* t = np[s] + (c * N + m) * 2 * ns[s];
-                J[s] = align(v[s], aK[s]) - align(t[0], aN[s]);
+                J[s] = align(v[s], aK[s][c]) - align(t[0], aN[s][c]) + jm;
                 O[s] = d[s];
                 Dn[s] = t[ns[s]];
                 if (normal) {
                     for (int mm = m - 1; mm >= 0; mm -= 2)
-                        x += align(op[s][((1 - DIR) * N + mm) * 2 * L::EP], aK[s]) -
-                             align(np[s][((1 - DIR) * N + mm) * 2 * ns[s]], aN[s]);
+                        x += align(op[s][(tc * N + mm) * 2 * L::NEL], aK[s][tc]) -
+                             align(np[s][(tc * N + mm) * 2 * ns[s]], aN[s][tc]);
                 } else {
                     for (int mm = m + 1; mm < N; mm += 2) {
-                        x += op[s][(DIR * N + mm) * 2 * L::EP];
+                        x += op[s][(DIR * N + mm) * 2 * L::NEL];
                         xn += np[s][(DIR * N + mm) * 2 * ns[s]];
                     }
                 }
@@ -488,18 +603,16 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
                 // Neumann (2) all so that nothing remains;
                 // Dirichlet (3) both values odd, both derivatives even
                 const bool on = kind[s] == 3 || (kind[s] == 1 && normal);
-                J[s] = on ? v[s] << 1 : 0;
-                O[s] = 0;
-                Dn[s] = on ? d[s] : 0;
-                if (on) O[s] = d[s];
+                J[s] = on ? (align(v[s], aK[s][c]) << 1) + jm : 0;
+                O[s] = on ? d[s] : 0;
+                Dn[s] = O[s];
                 if (kind[s] == 3) {
                     if (normal) {
                         for (int mm = m - 1; mm >= 0; mm -= 2)
-                            x += op[s][((1 - DIR) * N + mm) * 2 * L::EP];
-                        x <<= 1;
+                            x += align(op[s][(tc * N + mm) * 2 * L::NEL], aK[s][tc]) << 1;
                     } else {
                         for (int mm = m + 1; mm < N; mm += 2)
-                            x += op[s][(DIR * N + mm) * 2 * L::EP];
+                            x += op[s][(DIR * N + mm) * 2 * L::NEL];
                         xn = x;
                     }
                 }
@@ -522,7 +635,7 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
         if constexpr (DIR == 1) {   // second half of the cross volume terms
             i64 w[N];
 #pragma unroll
-            for (int j = 0; j < N; ++j) w[j] = sc[((1 - c) * L::NN + j * N + m) * L::EP + el];
+            for (int j = 0; j < N; ++j) w[j] = sc[((1 - c) * L::NN + j * N + m) * L::NEL + el];
             if (c == 0) {
 #pragma unroll
                 for (int b = 0; b < N; ++b) T[b] = b >= 1 ? (b >= 2 ? T[b - 2] : 0) + w[b - 1] : 0;
@@ -534,24 +647,29 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
         }
         // unit 2^om (on the grid of exponent E) of this line's W: the largest of its
         // terms (magnitude times factor and viscosity, number of terms of the kind)
-        // stays below 2^59, their sum below 2^62
-        unsigned bG = mag(O[0]) | mag(O[1]), bT = 0;
+        // stays below 2^59, their sum below 2^62.  Zeros of the other component do not
+        // count: on the grid of a large one they would coarsen what a small one gives.
+        unsigned bG = mag(O[0]) | mag(O[1]);
+        i64 nT = 0;
+        unsigned bT = 0;
 #pragma unroll
         for (int a = 1; a < N; ++a) bG |= mag(G[a]);
         if constexpr (DIR == 1) {
 #pragma unroll
-            for (int a = 0; a < N; ++a) bT |= mag(T[a]);
+            for (int a = 0; a < N; ++a) {
+                bT |= mag(T[a]);
+                nT |= T[a];
+            }
         }
-        int wb = imax(bit_length(bG) + ek, bit_length(bT)) + 2 - oK - rK;
-        int lJ[2], oX[2];
+        int wb = imax(bit_length(bG) + ek - oK[c], (nT == 0 ? NONE : bit_length(bT)) - oK[1 - c]) + 2 - rK;
+        int lJ[2];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             lJ[s] = bit_length(mag(J[s]));
-            oX[s] = normal ? oF[s] : oK;
-            wb = imax(wb, lJ[s] + imax(ep, ek + B::TRI) + 2 - oF[s] - rP[s]);
-            wb = imax(wb, bit_length(mag(Dn[s])) + ek + 2 - oN[s] - rN[s]);
-            wb = imax(wb, bit_length(mag(X[s])) + 2 - oX[s] - rK);
-            wb = imax(wb, bit_length(mag(Xn[s])) + 2 - oN[s] - rN[s]);
+            wb = imax(wb, lJ[s] + imax(ep, ek + B::TRI) + 2 - oG[s][c] - rP[s]);
+            wb = imax(wb, bit_length(mag(Dn[s])) + ek + 2 - oN[s][c] - rN[s]);
+            wb = imax(wb, length(X[s]) + 2 - oX[s] - rK);
+            wb = imax(wb, length(Xn[s]) + 2 - oN[s][DIR] - rN[s]);
         }
         const int om = wb + 32 + 3 - 62;
         // a high product of a term and a 62-bit mantissa is term * mantissa / 4
@@ -560,16 +678,16 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
         for (int s = 0; s < 2; ++s) {
             // jumps are small next to the traces where the field is smooth: shifted up
             // by what their magnitude leaves before they meet the large factors
-            const int js = 30 - lJ[s] > 0 ? 30 - lJ[s] : 0;
+            const int js = imax(30 - lJ[s], 0);
             const i64 j = J[s] << js;
-            i64 p = prod(O[s], wK, shift_by(om - 2 - ek + rK + half + oK)) +
-                    prod(Dn[s], wN[s], shift_by(om - 2 - ek + rN[s] + half + oN[s]));
+            i64 p = prod(O[s], wK, shift_by(om - 2 - ek + rK + half + oK[c])) +
+                    prod(Dn[s], wN[s], shift_by(om - 2 - ek + rN[s] + half + oN[s][c]));
             p += prod(X[s], wC, shift_by(om - 2 + rK + oX[s]));
-            if (!normal) p += prod(Xn[s], wCN[s], shift_by(om - 2 + rN[s] + oN[s]));
-            P[s] = prod(j, wP[s], shift_by(om - 2 + js - ep + rP[s] + oF[s])) + (s ? -p : p);
-            Q[s] = prod(j, wK, shift_by(om - 2 + js - ek + rK + half + oF[s]));
+            if (!normal) p += prod(Xn[s], wCN[s], shift_by(om - 2 + rN[s] + oN[s][DIR]));
+            P[s] = prod(j, wP[s], shift_by(om - 2 + js - ep + rP[s] + oG[s][c])) + (s ? -p : p);
+            Q[s] = prod(j, wK, shift_by(om - 2 + js - ek + rK + half + oG[s][c]));
         }
-        const Shift sG = shift_by(om - 4 - ek + rK + half + oK), sT = shift_by(om - 4 + rK + oK);
+        const Shift sG = shift_by(om - 4 - ek + rK + half + oK[c]), sT = shift_by(om - 4 + rK + oK[1 - c]);
         const i64 Pp = P[1] + P[0], Pm = P[1] - P[0];
         const i64 Qp = Q[1] + Q[0], Qm = Q[1] - Q[0];
 #pragma unroll
@@ -583,7 +701,7 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
                 W += prod(T[a], wC, sT);
                 // both parts to the coarser of their units
                 const int ur = unit[(c * N + a) * L::NEL + el], u = imax(ur, om);
-                W = align(W, shift_by(u - om)) + align(sw[mode * L::EP + el], shift_by(u - ur));
+                W = align(W, down_by(u - om)) + align(sw[mode * L::EP + el], down_by(u - ur));
                 // y = alpha s_a s_b W 2^(E - 1022 + ref + u - FRAC)
                 const double f = scale2(os[a * N + m], E - 1022 + ref + u - B::FRAC);
                 sw[mode * L::EP + el] = bits_of(W == 0 ? 0.0 : to_fp(W) * f);
@@ -601,12 +719,12 @@ FIX_HD void phase_lines(int tid, const Mesh& g, const Scal& k, const double* os,
                 for (int a = 0; a < N; ++a) q[a] = a >= 1 ? (a >= 2 ? q[a - 2] : 0) + U[a - 1] : 0;
             }
 #pragma unroll
-            for (int a = 0; a < N; ++a) sc[(c * L::NN + m * N + a) * L::EP + el] = q[a];
+            for (int a = 0; a < N; ++a) sc[(c * L::NN + m * N + a) * L::NEL + el] = q[a];
         }
     }
 }
 
-// Factor of entry q's conversion: s_i s_j 2^FRAC / 2^e_K.
+// Factor of an entry's conversion: s_i s_j 2^FRAC / 2^e.
 template <int N>
 FIX_HD double in_factor(double ss, int e) {
     return scale2(ss, Bound<N>::FRAC - (e - 1022));
