@@ -146,12 +146,16 @@ sip_status sip_problem_sizes(const sip_problem* prob, int64_t* n_u, int64_t* n_p
  * on the device and keeps the fastest; later problems of the same shape reuse
  * the choice.  apply[0] / apply[1]: SIP apply kernel of the FP64 / FP32
  * operator: 1 component-split thread pair per element, 2 one thread per
- * element, 3 shared-memory tile, 4 / 5 component-split thread pair on
- * element blocks staged through shared memory with 2 / 4 tile rows, 6 (FP32
- * operator only) one thread per element and one warp per tile row on
- * element blocks staged with asynchronous 16-byte copies.  An FP32 operator
- * with split-precision tiles (see mixed_fp64_ratio) reports 4: its marked
- * tiles run the staged kernel with FP64 arithmetic, the others kernel 6;
+ * element, 3 shared-memory tile, 4 (FP64) 64-bit fixed point on the integer
+ * pipes (values outside its range: FP64 formulas; meshes outside its range:
+ * the staged kernel), 4 (FP32) / 5 component-split thread pair on element
+ * blocks staged through shared memory with 2 / 4 tile rows, 6 (FP32 operator
+ * only) one thread per element and one warp per tile row on element blocks
+ * staged with asynchronous 16-byte copies.  An FP32 operator with
+ * split-precision tiles (see mixed_fp64_ratio) reports 4: its marked tiles run
+ * with FP64 accuracy (fixed point, or the staged kernel with FP64 arithmetic),
+ * the others kernel 6.  A Stokes solve of viscosity contrast above 128 runs
+ * its own choice among the kernels with FP64 arithmetic, which is not reported;
  * fused[0] / fused[1]: 1 if a p-level smoother step is one launch (apply,
  * block-Jacobi and Chebyshev update together), 0 if it is the apply and
  * block-Jacobi launches.  Either array may be NULL; the values are those of
@@ -160,7 +164,9 @@ sip_status sip_problem_schedule(const sip_problem* prob, int apply[2], int fused
 /* Pin the kernel schedule of this problem (no counterpart in the paper):
  * apply[t] in 0..6 with the codes of sip_problem_schedule (0 = autotuned;
  * 1, 2, 4, 5, 6 need k <= 5; 6 only for apply[1]), fused[t] in -1..1 (-1 = autotuned; 1 takes effect
- * only for k <= 3).  Either array may be NULL (unchanged).  The operator
+ * only for k <= 3).  Either array may be NULL (unchanged).  With a pinned
+ * kernel of FP64 arithmetic (apply[0] = 1, 2, 3, 5) B and B^T run as in a
+ * Stokes solve of high contrast, one thread per mode, too.  The operator
  * entry points use a pinned apply kernel at once; the multigrid set-up is
  * marked stale, so the next call that needs it rebuilds it (in the buffers
  * already held) with the pinned kernels.  Errors: INVALID_ARG. */

@@ -118,8 +118,9 @@ class Problem:
 
     def schedule(self):
         """sip_problem_schedule: {"apply": [fp64, fp32], "fused": [fp64, fp32]}
-        (apply: 1 component split, 2 one thread per element, 3 tile, 4 / 5
-        staged tile with 2 / 4 rows)."""
+        (apply: 1 component split, 2 one thread per element, 3 tile, 4 fixed
+        point (FP64) / staged tile with 2 rows (FP32), 5 staged tile with 4
+        rows, 6 warp row (FP32))."""
         apply = (ctypes.c_int * 2)()
         fused = (ctypes.c_int * 2)()
         self.ctx.check(self.ctx.lib.sip_problem_schedule(self.handle, apply, fused))

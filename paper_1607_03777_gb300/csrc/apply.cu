@@ -498,8 +498,13 @@ void launch_apply_sip(int N, const OpGeom& g, const T* x, T* y, const T* eta, T 
                                   reinterpret_cast<const float*>(z), float(beta), nullptr, s))
             return;
     }
-    // the FP64 operator's default is the staged entry too (fixed-point kernel)
-    if ((v == APPLY_STAGE || split || (sizeof(T) == 8 && v == APPLY_AUTO && !g.fp64)) &&
+    bool fix = false;
+    if constexpr (sizeof(T) == 8) {
+        fix = fixed_point(g, v);
+        if (fix && launch_apply_fix(N, g, x, y, eta, alpha, z, beta, nullptr, s)) return;
+    }
+    // factors outside the fixed-point range (meshes of extreme aspect): the staged kernel
+    if ((v == APPLY_STAGE || split || fix) &&
         launch_apply_sip_stage<T>(N, g, x, y, eta, alpha, z, beta, nullptr, s))
         return;
     if constexpr (sizeof(T) == 4) {

@@ -539,9 +539,6 @@ void stage_dispatch(const OpGeom& g, const T* x, T* y, const T* eta, T alpha, co
             stage_split<N>(g, x, y, eta, alpha, z, beta, r1, s);
             return;
         }
-    } else {
-        // FP64: the fixed-point kernel wherever it applies
-        if (!g.fp64 && launch_apply_fix(N, g, x, y, eta, alpha, z, beta, r1, s)) return;
     }
     if constexpr (StageLayout<N, T, T, 4>::BYTES <= kMaxSmem) {
         if (g.stage_rows[sizeof(T) == 4 ? 1 : 0] == 4) {

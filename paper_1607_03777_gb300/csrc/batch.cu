@@ -811,6 +811,7 @@ void BatchEngine<T>::build(cudaStream_t s) {
             sip_problem* P = probs[m];
             Multigrid<T>& G = mg(P);
             const BMember<T>& b = hm[m];
+            g.fix = g.fix && !P->geom.fp64;
             const T* eta = sizeof(T) == 4 ? reinterpret_cast<const T*>(P->eta_f.ptr)
                                           : reinterpret_cast<const T*>(P->eta_d.ptr);
             const T* eta_inv = sizeof(T) == 4 ? reinterpret_cast<const T*>(P->eta_inv_f.ptr)

@@ -229,9 +229,9 @@ sip_status sip_problem_schedule(const sip_problem* p, int apply[2], int fused[2]
     for (int t = 0; t < 2; ++t) {
         if (apply) {
             const int v = p->geom.variant[t];
-            apply[t] = v != sip::APPLY_AUTO ? v : (p->n <= 6 ? int(t == 0 ? sip::APPLY_STAGE : sip::APPLY_ELEM2)
-                                                             : int(sip::APPLY_TILE));
-            if (apply[t] == int(sip::APPLY_STAGE) && p->geom.stage_rows[t] == 4) apply[t] = 5;
+            if (t == 0 && p->n <= 6 && sip::fixed_point(p->geom, v)) apply[t] = 4;
+            else if (v == sip::APPLY_STAGE) apply[t] = t == 0 || p->geom.stage_rows[t] == 4 ? 5 : 4;
+            else apply[t] = v != sip::APPLY_AUTO ? v : int(p->n <= 6 ? sip::APPLY_ELEM2 : sip::APPLY_TILE);
             if (t == 1 && p->geom.n_hi > 0 && p->n <= 6) apply[t] = int(sip::APPLY_STAGE);
         }
         if (fused) fused[t] = (p->n <= 4 && p->geom.fused[t]) ? 1 : 0;
@@ -257,10 +257,8 @@ sip_status sip_problem_set_schedule(sip_problem* p, const int apply[2], const in
         if (apply) {
             p->pin_apply[t] = apply[t];
             if (apply[t] > 0) {
-                for (sip::OpGeom* g : {&p->geom, &p->geom_solve}) {
-                    g->variant[t] = apply[t] == 5 ? int(sip::APPLY_STAGE) : apply[t];
-                    g->stage_rows[t] = apply[t] == 5 ? 4 : 2;
-                }
+                sip::set_apply_code(p->geom, t, apply[t]);
+                p->pin_solve(t);
             }
         }
         if (fused) {

@@ -106,8 +106,6 @@ int fix_tile_count(int nx, int ny);
 template <typename TS>
 void launch_apply_fix_batch(int N, const FixArgs<TS>* args, const int2* items, int n_items,
                             const int* active, cudaStream_t s);
-bool launch_apply_fix(int N, const OpGeom& g, const double* x, double* y, const double* eta,
-                      double alpha, const double* z, double beta, double* r1, cudaStream_t s);
 // the tiles of g.hi_tiles only
 bool launch_apply_fix_list(int N, const OpGeom& g, const float* x, float* y, const float* eta,
                            float alpha, const float* z, float beta, float* r1, cudaStream_t s);

@@ -148,19 +148,24 @@ Tab1D<N, T> make_tab() {
 // Kernel schedule of one operator, per precision ([0] FP64, [1] FP32):
 // which apply kernel runs and whether the p-level smoother step is fused.
 // APPLY_WARP exists for the FP32 operator only (one thread per element, one
-// warp per tile row, cp.async staging).
+// warp per tile row, cp.async staging), APPLY_FIX for the FP64 one (fixed point,
+// apply_fix.cu).
 enum ApplyVariant { APPLY_AUTO = 0, APPLY_ELEM2 = 1, APPLY_ELEM1 = 2, APPLY_TILE = 3, APPLY_STAGE = 4,
-                    APPLY_WARP = 6 };
+                    APPLY_WARP = 6, APPLY_FIX = 7 };
 
 struct OpGeom {
     int nx, ny;
     double hx, hy;
     int bc[4];
     double pen_x, pen_y;
-    int variant[2];   // ApplyVariant (APPLY_AUTO: component-split for N <= 6, else tile)
+    // ApplyVariant (APPLY_AUTO: FP64 fixed point unless fp64 is set, else component-split,
+    // for N <= 6; above the tile kernel)
+    int variant[2];
     int fused[2];     // p-level smoother step fused into one launch (1) or not (0)
     int stage_rows[2];   // tile rows of the staged apply (2 or 4), per precision
-    int fp64;   // 1: the FP64 operator, B and B^T in FP64 arithmetic throughout (solve_geom)
+    // 1: the kernels of FP64 arithmetic throughout: no fixed point in the FP64 operator,
+    // B and B^T one thread per mode (sip_problem::geom_solve, pinned FP64 kernels)
+    int fp64;
     // split-precision FP32 operator (mixed form at high viscosity contrast):
     // tiles evaluated in FP64 arithmetic on FP32 data; n_hi = 0: none
     const unsigned char* hi_flag;
@@ -189,11 +194,24 @@ inline OpGeom make_geom(int nx, int ny, double lx, double ly, const int bc[4], i
     return g;
 }
 
+// Schedule code `code` > 0 of sip_problem_set_schedule for precision t.
+inline void set_apply_code(OpGeom& g, int t, int code) {
+    g.variant[t] = code == 5 ? int(APPLY_STAGE) : (code == 4 && t == 0 ? int(APPLY_FIX) : code);
+    g.stage_rows[t] = code == 5 ? 4 : 2;
+    if (t == 0) g.fp64 = code != 4;
+}
+// The FP64 operator runs in fixed point under variant v.
+inline bool fixed_point(const OpGeom& g, int v) { return v == APPLY_FIX || (v == APPLY_AUTO && !g.fp64); }
+
 // y = alpha * (A x) + beta * z (z may be null).  N = polynomial degree + 1
 // of the space the operator acts on (N = 2 for the Galerkin A_1).
 template <typename T>
 void launch_apply_sip(int N, const OpGeom& g, const T* x, T* y, const T* eta, T alpha,
                       const T* z, T beta, cudaStream_t s);
+// The FP64 operator in fixed point (apply_fix.cu); r1 non-null: only the Q^2_1 modes of the
+// result, there.  Returns false where it does not apply (degree, factors out of range).
+bool launch_apply_fix(int N, const OpGeom& g, const double* x, double* y, const double* eta,
+                      double alpha, const double* z, double beta, double* r1, cudaStream_t s);
 // Thread-per-element variants for N <= 6 (split: two threads per element,
 // one per velocity component); returns false for other N.
 template <typename T>

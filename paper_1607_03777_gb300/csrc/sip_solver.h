@@ -344,6 +344,12 @@ struct sip_problem {
     bool contrast_known = false;   // stiff belongs to the present viscosities
     bool in_stokes = false;        // a stiff problem's Stokes solve is running
     const sip::OpGeom& op() const { return in_stokes ? geom_solve : geom; }
+    // the pinned kernel of precision t in geom_solve: for the fixed-point one the staged
+    void pin_solve(int t) {
+        sip::set_apply_code(geom_solve, t, pin_apply[t]);
+        if (geom_solve.variant[t] == sip::APPLY_FIX) geom_solve.variant[t] = sip::APPLY_STAGE;
+        geom_solve.fp64 = 1;
+    }
     sip::OpGeom geom1{};     // the Galerkin Q_1 operator (fine-k penalty)
     std::vector<double> eta_host;
     sip::DeviceBuffer eta_d, eta_f, eta_inv_d, eta_inv_f;

@@ -6,8 +6,10 @@
 // covers every degree, and the staged-tile kernel (element blocks copied
 // through shared memory with coalesced 16-byte accesses, 2 or 4 tile rows)
 // suits the memory-bound FP32 operator, as does the warp-row kernel (one
-// thread per element, one warp per tile row, cp.async staging; FP32 only).  So each problem times the candidates on its own mesh
-// the first time it is set up and keeps the fastest:
+// thread per element, one warp per tile row, cp.async staging; FP32 only), and
+// the fixed-point kernel (FP64 only) takes the FP64 operator's products to the
+// integer pipes.  So each problem times the candidates on its own mesh the
+// first time it is set up and keeps the fastest:
 //   * the apply kernel, per precision the problem runs in;
 //   * the p-level smoother step: one fused launch (apply + block-Jacobi +
 //     Chebyshev update) against the apply and block-Jacobi launches.
@@ -102,8 +104,8 @@ void tune_apply_t(sip_problem* P, OpGeom& g, cudaStream_t s) {
         const int64_t launches = launch_counter();
         const int saved_rows = g.stage_rows[t];
         for (int cand : {int(APPLY_ELEM2), int(APPLY_ELEM1), int(APPLY_TILE),
-                         int(APPLY_STAGE) + 16 * 2, int(APPLY_STAGE) + 16 * 4,
-                         sizeof(T) == 4 ? int(APPLY_WARP) : -1}) {
+                         sizeof(T) == 8 && !g.fp64 ? int(APPLY_FIX) : int(APPLY_STAGE) + 16 * 2,
+                         int(APPLY_STAGE) + 16 * 4, sizeof(T) == 4 ? int(APPLY_WARP) : -1}) {
             if (cand < 0) continue;
             g.variant[t] = cand % 16;
             g.stage_rows[t] = cand / 16 ? cand / 16 : saved_rows;
@@ -130,16 +132,17 @@ void tune_apply_t(sip_problem* P, OpGeom& g, cudaStream_t s) {
 
 void tune_apply(sip_problem* P, cudaStream_t s) {
     for (int t = 0; t < 2; ++t)
-        if (P->pin_apply[t] > 0) {   // pinned: code 5 = staged with 4 tile rows
-            P->geom.variant[t] = P->pin_apply[t] == 5 ? int(APPLY_STAGE) : P->pin_apply[t];
-            P->geom.stage_rows[t] = P->pin_apply[t] == 5 ? 4 : 2;
-        }
+        if (P->pin_apply[t] > 0)
+            set_apply_code(P->geom, t, P->pin_apply[t]);
+        else if (t == 0)
+            P->geom.fp64 = 0;
     // one kernel exists above degree 5
     const bool on = autotune_on() && P->n <= 6;
     if (on && P->pin_apply[0] == 0) tune_apply_t<double>(P, P->geom, s);
     if (on && P->pin_apply[1] == 0 && P->desc.precision != SIP_PREC_FP64) tune_apply_t<float>(P, P->geom, s);
     P->geom_solve = P->geom;
     P->geom_solve.fp64 = 1;
+    if (P->pin_apply[0] > 0) P->pin_solve(0);
     if (!P->stiff || P->pin_apply[0] > 0) return;
     P->geom_solve.variant[0] = APPLY_AUTO;
     P->geom_solve.stage_rows[0] = 2;
