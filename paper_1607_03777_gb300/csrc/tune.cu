@@ -91,7 +91,8 @@ double time_ms(F&& f, cudaStream_t s, int reps) {
 template <typename T>
 void tune_apply_t(sip_problem* P, OpGeom& g, cudaStream_t s) {
     const int t = sizeof(T) == 4 ? 1 : 0;
-    const Key key{g.fp64 ? 2 : 0, P->n, int(sizeof(T)), P->desc.nx, P->desc.ny};
+    // the FP64 operator's choices per arithmetic; FP32 ones are the same in both schedules
+    const Key key{sizeof(T) == 8 && g.fp64 ? 2 : 0, P->n, int(sizeof(T)), P->desc.nx, P->desc.ny};
     int best = APPLY_AUTO;   // variant + 16 x stage rows
     if (!cached(key, best)) {
         const size_t n_u = size_t(P->n_u);
@@ -157,7 +158,7 @@ void Multigrid<T>::tune_smoother(OpGeom& g, cudaStream_t s) {
         return;
     }
     if (!autotune_on() || !cheb_elem_available(N) || !pd2.ptr) return;
-    const Key key{g.fp64 ? 3 : 1, N, int(sizeof(T)), P->desc.nx, P->desc.ny};
+    const Key key{sizeof(T) == 8 && g.fp64 ? 3 : 1, N, int(sizeof(T)), P->desc.nx, P->desc.ny};
     int fused = 1;
     if (!cached(key, fused)) {
         T* b = pb.template as<T>();
@@ -195,11 +196,12 @@ void Multigrid<T>::tune_smoother(OpGeom& g, cudaStream_t s) {
 
 template <typename T>
 void Multigrid<T>::tune_smoother(cudaStream_t s) {
+    const int t = sizeof(T) == 4 ? 1 : 0;
     tune_smoother(P->geom, s);
     if (sizeof(T) == 8 && P->stiff)
         tune_smoother(P->geom_solve, s);
-    else
-        for (int t = 0; t < 2; ++t) P->geom_solve.fused[t] = P->geom.fused[t];
+    else   // this precision's entry: the other's belongs to its own set-up
+        P->geom_solve.fused[t] = P->geom.fused[t];
 }
 
 template void Multigrid<double>::tune_smoother(cudaStream_t);
