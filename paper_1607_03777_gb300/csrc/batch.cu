@@ -571,8 +571,10 @@ struct BatchEngine {
     int maxit = 0;
     int steps_p = 0, steps_h = 0;
     DeviceBuffer d_mem, d_state, d_act, d_partial;
-    // per degree N: apply role tables (V-cycle precision, plus the FP64-
-    // arithmetic tiles of split members) and their work lists
+    // per degree N, members held to FP64 arithmetic (viscosity contrast above
+    // sip_problem::kFixedContrast, or a pinned FP64 kernel) apart: apply role tables
+    // (V-cycle precision, plus the FP64-arithmetic tiles of split members) and their work
+    // lists
     struct Group {
         int N = 0;
         // operator roles: dec0 pr = vin - A pd (first step from zero), dec pr -= A pd,
@@ -585,7 +587,7 @@ struct BatchEngine {
         std::vector<DeviceBuffer> bj;   // block-Jacobi tables: [0] first step pre, [1] first step post, [1 + st] step st
     };
     std::vector<Group> groups;
-    // degrees run side by side within a stage: a stream per further group
+    // groups run side by side within a stage: a stream per further one
     std::vector<cudaStream_t> side;
     std::vector<cudaEvent_t> ev;
     // continuous levels in two launches each (hlevel.cu), where every level allows it
@@ -617,7 +619,7 @@ struct BatchEngine {
         for (cudaStream_t t : side) cudaStreamDestroy(t);
         for (cudaEvent_t t : ev) cudaEventDestroy(t);
     }
-    // f(group, stream) for every degree: the first on s, the others beside it
+    // f(group, stream) for every group: the first on s, the others beside it
     template <class F>
     void each_group(cudaStream_t s, F f) {
         const size_t n = groups.size();
@@ -784,12 +786,15 @@ void BatchEngine<T>::build(cudaStream_t s) {
             throw Error(SIP_ERR_OOM, "pinned host allocation failed");
         }
     }
-    // element kernels, per degree
+    // element kernels, per degree and arithmetic.  A stiff member's inner solves keep the
+    // FP64 kernels as run_solve does, for the same reason (sip_problem::geom_solve).
     groups.clear();
-    for (int N = 2; N <= 6; ++N) {
+    for (int id = 0; id < 10; ++id) {
+        const int N = 2 + id / 2;
+        const bool fp64 = id % 2 == 1;
         std::vector<int> ms;
         for (int m = 0; m < nmem; ++m)
-            if (probs[m]->n == N) ms.push_back(m);
+            if (probs[m]->n == N && (probs[m]->stiff || probs[m]->geom.fp64) == fp64) ms.push_back(m);
         if (ms.empty()) continue;
         Group g;
         g.N = N;
@@ -803,7 +808,7 @@ void BatchEngine<T>::build(cudaStream_t s) {
         }
         std::vector<StageArgs<double, double>> qa(nmem);
         std::vector<FixArgs<double>> fq(nmem);
-        g.fix = true;
+        g.fix = !fp64;
         std::vector<int2> lo, hi, all, fixed, bjit;
         const int nbj = steps_p + 1;
         std::vector<std::vector<BJBatchArgs<T>>> bjt(nbj, std::vector<BJBatchArgs<T>>(nmem));
@@ -811,7 +816,6 @@ void BatchEngine<T>::build(cudaStream_t s) {
             sip_problem* P = probs[m];
             Multigrid<T>& G = mg(P);
             const BMember<T>& b = hm[m];
-            g.fix = g.fix && !P->geom.fp64;
             const T* eta = sizeof(T) == 4 ? reinterpret_cast<const T*>(P->eta_f.ptr)
                                           : reinterpret_cast<const T*>(P->eta_d.ptr);
             const T* eta_inv = sizeof(T) == 4 ? reinterpret_cast<const T*>(P->eta_inv_f.ptr)

@@ -38,3 +38,31 @@ def test_fp32_setup_keeps_the_choice(ctx, n, k):
     x = torch.as_tensor(synth.random_vector(Q.n_u, 3)).float().cuda()
     Q.vcycle_f32(x, torch.empty_like(x))
     assert torch.equal(solve(P, f), solve(Q, f))
+
+
+def grouped(ctx, members):
+    """Grouped batch of (problem, load vector) pairs; the solutions."""
+    fs = [f for _, f in members]
+    us = [torch.empty_like(f) for f in fs]
+    ps = [torch.empty(P.n_p, dtype=torch.float64, device="cuda") for P, _ in members]
+    st, reps = api.solve_batch(ctx, [P for P, _ in members], fs, us, ps, n_streams=len(members), rtol=1e-8,
+                               grouped=True)
+    assert st == 0 and all(r["rel_residual"] <= 1e-8 for r in reps)
+    return [torch.cat([u, p]) for u, p in zip(us, ps)]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("k", [2, 3])
+def test_grouped_stiff_members(ctx, precision, k):
+    """Stiff members of a grouped batch run the FP64 kernels: their bits are those of one of
+    the pinned kernels (outer operator and set-up follow the pin, the inner loop is the
+    same).  Members of low contrast do not depend on them."""
+    contrasts = (1e3, 1e4, 1e2)
+
+    def run(code, which=contrasts):
+        return grouped(ctx, [problem(ctx, 32, k, c, precision, code) for c in which])
+
+    got, pinned = run(0), [run(code) for code in (1, 2, 3, 5)]
+    for m in (0, 1):
+        assert any(torch.equal(got[m], p[m]) for p in pinned), contrasts[m]
+    assert torch.equal(got[2], run(0, (1e2, 50.0))[0])
