@@ -504,8 +504,9 @@ ForkStream& fork_stream() {
 
 // Split-precision FP32 apply: FP32 arithmetic on the tiles not flagged in
 // g.hi_flag, FP64 arithmetic on the g.n_hi tiles of g.hi_tiles.  The FP64
-// launch has few CTAs and runs at the FP64 pipe's rate; the FP32 launch
-// fills the SMs beside it on a second stream.
+// launch has few CTAs and runs at the FP64 pipe's rate (or, but in stiff Stokes
+// solves, in fixed point at the integer pipes'); the FP32 launch fills the SMs
+// beside it on a second stream.
 template <int N>
 void stage_split(const OpGeom& g, const float* x, float* y, const float* eta, float alpha,
                  const float* z, float beta, float* r1, cudaStream_t s) {
@@ -516,7 +517,7 @@ void stage_split(const OpGeom& g, const float* x, float* y, const float* eta, fl
     hi.tiles = g.hi_tiles;
     SIP_CUDA(cudaEventRecord(f.fork, s));
     SIP_CUDA(cudaStreamWaitEvent(f.s, f.fork, 0));
-    if (!launch_apply_fix_list(N, g, x, y, eta, alpha, z, beta, r1, f.s))
+    if (g.fp64 || !launch_apply_fix_list(N, g, x, y, eta, alpha, z, beta, r1, f.s))
         launch_stage<N, float, double, SPLIT_TYS, true>(hi, dim3(unsigned(g.n_hi)), vec, f.s);
     SIP_CUDA(cudaEventRecord(f.join, f.s));
     // the unflagged tiles: the warp-row kernel (y = alpha A x + beta z), else

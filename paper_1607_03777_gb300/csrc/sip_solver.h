@@ -233,6 +233,8 @@ struct Multigrid {
     // r1 = R (b - A y) in one launch where a kernel for it exists
     bool residual_restrict(const T* y, const T* b, T* r1, cudaStream_t s);
     void build_coarse_from_band(const std::vector<double>& band, int n, int bw, cudaStream_t s);
+    bool own_schedule() const;
+    void replay(cudaStream_t s);
 };
 
 // Graph-resident inner PCG (inner_graph.cu).

@@ -898,17 +898,34 @@ void Multigrid<T>::vcycle_on(const T* b, T* y, cudaStream_t s) {
     smooth_p(b, y, false, s);
 }
 
+// A stiff Stokes solve runs kernels that the graph does not hold (FP32: in marked tiles
+// only).  Launched one by one they take no longer: 128^2, k = 3, host-driven inner loop
+// 138 ms a solve, 139 from a second graph; 32^2, k = 2 34 and 35 ms.
+template <typename T>
+bool Multigrid<T>::own_schedule() const {
+    return P->in_stokes && (sizeof(T) == 8 || n_hi > 0);
+}
+
+// vin -> vout by the schedule in force
+template <typename T>
+void Multigrid<T>::replay(cudaStream_t s) {
+    if (own_schedule()) {
+        vcycle_direct(s);
+        return;
+    }
+    SIP_CUDA(cudaGraphLaunch(graph, s));
+    launch_counter() += graph_kernels;
+}
+
 template <typename T>
 void Multigrid<T>::vcycle(const T* r, T* z, cudaStream_t s) {
-    // the graph holds the other schedule's kernels (FP32: the same in both)
-    if (sizeof(T) == 8 && P->in_stokes && r != z) {
+    if (own_schedule() && r != z) {
         vcycle_on(r, z, s);
         return;
     }
     if (r != vin.template as<T>())
         SIP_CUDA(cudaMemcpyAsync(vin.ptr, r, n_u * sizeof(T), cudaMemcpyDeviceToDevice, s));
-    SIP_CUDA(cudaGraphLaunch(graph, s));
-    launch_counter() += graph_kernels;
+    replay(s);
     if (z != vout.template as<T>())
         SIP_CUDA(cudaMemcpyAsync(z, vout.ptr, n_u * sizeof(T), cudaMemcpyDeviceToDevice, s));
 }
@@ -963,8 +980,7 @@ int Multigrid<T>::inner_pcg(const T* t, T* y, double rtol, int maxit, cudaStream
 template <typename T>
 void Multigrid<T>::vcycle_widen(const double* r, double* z, cudaStream_t s) {
     launch_cast<double, T>(n_u, r, vin.template as<T>(), s);
-    SIP_CUDA(cudaGraphLaunch(graph, s));
-    launch_counter() += graph_kernels;
+    replay(s);
     launch_cast<T, double>(n_u, vout.template as<T>(), z, s);
 }
 

@@ -66,3 +66,35 @@ def test_grouped_stiff_members(ctx, precision, k):
     for m in (0, 1):
         assert any(torch.equal(got[m], p[m]) for p in pinned), contrasts[m]
     assert torch.equal(got[2], run(0, (1e2, 50.0))[0])
+
+
+@pytest.mark.parametrize("inner_loop", ["device", "host"])
+@pytest.mark.parametrize("k", [2, 3])
+def test_marked_tiles_of_the_fp32_cycle(ctx, k, inner_loop):
+    """Mixed form, contrast 1e5: the solve's FP32 cycle runs its marked tiles in FP64
+    arithmetic, so a run with pinned FP64 kernels has its bits; outside a solve they run in
+    fixed point unless an FP64 kernel is pinned."""
+    n = 32
+    P, f = problem(ctx, n, k, 1e5, "mixed")
+    got = solve(P, f, inner_loop=inner_loop)
+    pinned = []
+    for code in (1, 2, 3, 5):
+        Q, g = problem(ctx, n, k, 1e5, "mixed", code)
+        pinned.append(solve(Q, g, inner_loop=inner_loop))
+    assert any(torch.equal(got, p) for p in pinned)
+    # a linear field without strain: what remains inside is rounding, another in either form
+    m, h = k + 1, 1.0 / n
+    x = torch.zeros(n, n, 2, m, m, dtype=torch.float64)
+    at = (torch.arange(n, dtype=torch.float64) + 0.5) * h - 0.5
+    x[:, :, 0, 0, 0], x[:, :, 1, 0, 0] = -2.0 * at[:, None], 2.0 * at[None, :]
+    x[:, :, 0, 1, 0], x[:, :, 1, 0, 1] = -h / 3.0 ** 0.5, h / 3.0 ** 0.5
+    x = x.reshape(-1).float().cuda()
+    y = [torch.empty_like(x) for _ in range(3)]
+    for q, out in ((P, y[0]), (Q, y[1])):
+        q.apply_A_f32(x, out)
+    assert P.schedule()["apply"][1] == 4   # marked tiles
+    assert not torch.equal(y[0], y[1])
+    Q.set_schedule(apply=[4, 0])
+    Q.setup()
+    Q.apply_A_f32(x, y[2])
+    assert torch.equal(y[0], y[2])
