@@ -6,7 +6,13 @@
 // line) forms a line's scaled entries, their even and odd sums (both end
 // traces) and their prefix sums (int l_p l_q' = 2 l_p(1) l_q(1) for q > p, q - p
 // odd) once: about 35 FP64 operations per line at k = 4 instead of 230.
-// 250 x 190, k = 4, both operators: 417 us before.
+// 250 x 190, k = 4, both operators: 417 us before, 72 now.
+//
+// Mode q receives (h / 2) l_q(1) (f_1 - (-1)^q f_0 - 2 sum of the other parity beyond q) with
+// f_s = c_s own_s + neighbour_s / 2 and own_s = even +- odd sum.  In the traces' sum and
+// difference one parity cancels between the faces, so its coefficients c_1 +- c_0 are
+// formed first; with the sums by fused multiply-adds the error is below that of the
+// one-thread-per-mode kernels (the difference of rounded traces was above it).
 //
 // Layout: a CTA serves 32 elements of one mesh row, a warp per line, a lane per
 // element.  The row, its left and right neighbour and the rows below and above
@@ -21,16 +27,21 @@ namespace {
 
 constexpr int WX = 32;   // elements per CTA
 
+// sqrt(2 i + 1) = sqrt(2) l_i(1): without rounding for i = 0 and 4
+__device__ constexpr double kRoot[7] = {1.0, 1.7320508075688772, 2.23606797749979, 2.6457513110645907, 3.0,
+                             3.3166247903554, 3.605551275463989};
+
 struct DivArgs {
     const double* in;
     double* out;
     int nx, ny;
-    double hx, hy;
     int bc[4];
+    double hl[2][7];   // sqrt(2 q + 1) times a quarter of the face's length, per direction of the normal
 };
 
 // Rows ey - 1, ey, ey + 1 of a vector of NE entries per element, columns
-// ex0 - 1 .. ex0 + 32, into s[row][column][entry]; zeros outside the mesh.
+// ex0 - 1 .. ex0 + 32, into s[row][column][entry]; entries outside the mesh are left
+// unset and must not be read.
 template <int NE, int ES>
 __device__ __forceinline__ void load_rows(const DivArgs& a, int ex0, int ey, double* s) {
     const int lo = max(ex0 - 1, 0), hi = min(ex0 + WX + 1, a.nx);
@@ -47,14 +58,36 @@ __device__ __forceinline__ void load_rows(const DivArgs& a, int ex0, int ey, dou
 }
 
 // Weighted even and odd sums of a line: traces at the ends are ev + od, ev - od.
-template <int N, int L>
-__device__ __forceinline__ void even_odd(const double* p, int stride, double (&t)[L], double& ev, double& od) {
+template <int L>
+__device__ __forceinline__ void even_odd(const double* p, int stride, double& ev, double& od) {
     ev = od = 0.0;
 #pragma unroll
     for (int i = 0; i < L; ++i) {
-        t[i] = kT<N>.lp[i] * p[i * stride];
-        if (i % 2 == 0) ev += t[i]; else od += t[i];
+        double& a = i % 2 == 0 ? ev : od;
+        a = fma(kRoot[i], p[i * stride], a);
     }
+}
+
+// What a line's traces give to the modes of either parity (even: difference of the ends,
+// odd: sum), sg / 2 the neighbours' weight; nb entries to the neighbour on the plus side.
+template <int L>
+__device__ __forceinline__ void end_traces(const DivArgs& a, int dir, int ex, int ey, const double* p, int stride,
+                                           int nb, double sg, double& fe, double& fo) {
+    double ev, od, e2, o2, c[2], n[2];
+    even_odd<L>(p, stride, ev, od);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const bool in = dir == 0 ? (s ? ex < a.nx - 1 : ex > 0) : (s ? ey < a.ny - 1 : ey > 0);
+        n[s] = 0.0;
+        if (in) {
+            even_odd<L>(p + (s ? nb : -nb), stride, e2, o2);
+            n[s] = s ? e2 - o2 : e2 + o2;
+        }
+        c[s] = in ? 0.5 : (a.bc[2 * dir + s] == SIP_BC_NEUMANN ? 0.0 : 1.0);
+    }
+    const double cp = c[1] + c[0], cm = c[1] - c[0];
+    fe = fma(sg, n[1] - n[0], fma(cm, ev, cp * od));
+    fo = fma(sg, n[1] + n[0], fma(cm, od, cp * ev));
 }
 
 // B p: the N modes along the normal of line m (m < K) of component dir.
@@ -75,29 +108,17 @@ __global__ void __launch_bounds__(WX * 2 * (N - 1)) k_div_B(const DivArgs a) {
         const int stride = dir == 0 ? 1 : K, at = dir == 0 ? m * K : m;
         const double* p = sp + ((WX + 2) + lane + 1) * ES + at;
         const int nb = dir == 0 ? ES : (WX + 2) * ES;   // to the neighbour on the plus side
-        double t[K], u[K], ev, od, e2, o2;
-        even_odd<N, K>(p, stride, t, ev, od);
-        const double h = 0.5 * (dir == 0 ? a.hy : a.hx);
-        double f[2];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const bool in = dir == 0 ? (s ? ex < a.nx - 1 : ex > 0) : (s ? ey < a.ny - 1 : ey > 0);
-            const double own = s ? ev + od : ev - od;
-            if (in) {
-                even_odd<N, K>(p + (s ? nb : -nb), stride, u, e2, o2);
-                f[s] = 0.5 * h * (own + (s ? e2 - o2 : e2 + o2));
-            } else {
-                f[s] = a.bc[2 * dir + s] == SIP_BC_NEUMANN ? 0.0 : h * own;
-            }
-        }
-        const double fm = f[1] - f[0], fp = f[1] + f[0];
+        double fe, fo;
+        end_traces<K>(a, dir, ex, ey, p, stride, nb, 0.5, fe, fo);
         double* o = so + lane * OS + dir * NN + (dir == 0 ? m * N : m);
         double pe = 0.0, po = 0.0;   // sums of the even / odd entries below q
 #pragma unroll
         for (int q = 0; q < N; ++q) {
-            const double v = q % 2 == 0 ? fm - 2.0 * h * po : fp - 2.0 * h * pe;
-            o[dir == 0 ? q : q * N] = kT<N>.lp[q] * v;
-            if (q < K) (q % 2 == 0 ? pe : po) += t[q < K ? q : 0];
+            o[dir == 0 ? q : q * N] = a.hl[dir][q] * (q % 2 == 0 ? fma(-2.0, po, fe) : fma(-2.0, pe, fo));
+            if (q < K) {
+                double& b = q % 2 == 0 ? pe : po;
+                b = fma(kRoot[q], p[q * stride], b);
+            }
         }
     }
     __syncthreads();
@@ -126,27 +147,14 @@ __global__ void __launch_bounds__(WX * 2 * (N - 1)) k_div_Bt(const DivArgs a) {
         const int stride = dir == 0 ? 1 : N, at = dir * NN + (dir == 0 ? m * N : m);
         const double* u = su + ((WX + 2) + lane + 1) * ES + at;
         const int nb = dir == 0 ? ES : (WX + 2) * ES;
-        double t[N], w[N], ev, od, e2, o2;
-        even_odd<N, N>(u, stride, t, ev, od);
-        const double h = 0.5 * (dir == 0 ? a.hy : a.hx);
-        double f[2];
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const bool in = dir == 0 ? (s ? ex < a.nx - 1 : ex > 0) : (s ? ey < a.ny - 1 : ey > 0);
-            const double own = s ? ev + od : ev - od;
-            if (in) {
-                even_odd<N, N>(u + (s ? nb : -nb), stride, w, e2, o2);
-                f[s] = 0.5 * h * (own - (s ? e2 - o2 : e2 + o2));
-            } else {
-                f[s] = a.bc[2 * dir + s] == SIP_BC_NEUMANN ? 0.0 : h * own;
-            }
-        }
-        const double fm = f[1] - f[0], fp = f[1] + f[0];
+        double fe, fo;
+        end_traces<N>(a, dir, ex, ey, u, stride, nb, -0.5, fe, fo);
         double se = 0.0, so_ = 0.0;   // sums of the even / odd entries above q
 #pragma unroll
         for (int q = N - 1; q >= 0; --q) {
-            if (q < K) r[q < K ? q : 0] = kT<N>.lp[q] * (q % 2 == 0 ? fm - 2.0 * h * so_ : fp - 2.0 * h * se);
-            (q % 2 == 0 ? se : so_) += t[q];
+            if (q < K) r[q < K ? q : 0] = a.hl[dir][q] * (q % 2 == 0 ? fma(-2.0, so_, fe) : fma(-2.0, se, fo));
+            double& b = q % 2 == 0 ? se : so_;
+            b = fma(kRoot[q], u[q * stride], b);
         }
         if (dir == 0) {
 #pragma unroll
@@ -182,7 +190,15 @@ void launch_div(const DivArgs& a, cudaStream_t s) {
 
 template <bool TRANSPOSE>
 void launch_div_k(int k, const OpGeom& g, const double* in, double* out, cudaStream_t s) {
-    DivArgs a{in, out, g.nx, g.ny, g.hx, g.hy, {g.bc[0], g.bc[1], g.bc[2], g.bc[3]}};
+    DivArgs a{in, out, g.nx, g.ny, {g.bc[0], g.bc[1], g.bc[2], g.bc[3]}, {}};
+    for (int q = 0; q <= k; ++q) {
+        // the root with its rounding error, so that the products round once
+        const double x = 2.0 * q + 1.0, l = std::sqrt(x), d = std::fma(-l, l, x) / (2.0 * l);
+        for (int dir = 0; dir < 2; ++dir) {
+            const double h = 0.25 * (dir == 0 ? g.hy : g.hx);
+            a.hl[dir][q] = std::fma(h, l, h * d);
+        }
+    }
     switch (k + 1) {
         case 2: launch_div<2, TRANSPOSE>(a, s); break;
         case 3: launch_div<3, TRANSPOSE>(a, s); break;
