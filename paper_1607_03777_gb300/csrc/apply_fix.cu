@@ -327,7 +327,7 @@ void launch_tiles(const FixArgs<TS>& a, cudaStream_t s) {
 template <int N>
 void launch_mesh(const FixArgs<double>& a, cudaStream_t s) {
     constexpr int TW = N == 2 ? 16 : 8, TH = N <= 4 ? 8 : 4;
-    if (TH > 4 && (long long)((a.nx + TW - 1) / TW) * ((a.ny + TH - 1) / TH) < 152)
+    if (TH > 4 && (long long)((a.nx + TW - 1) / TW) * ((a.ny + TH - 1) / TH) < kSMs)
         launch_tiles<N, 8, 4, double>(a, s);
     else
         launch_tiles<N, TW, TH, double>(a, s);

@@ -46,7 +46,7 @@ template <typename T>
 struct BMember {
     int N, nx, ny, L;   // degree + 1, mesh, coarsest continuous level
     long long ne, n_u;
-    T *vin, *vout, *pr, *pd, *r1, *e1;
+    T *vin, *vout, *pr, *pd, *r1;
     int hnx[kMaxLv], hny[kMaxLv];   // elements per side of continuous level l
     long long hn[kMaxLv];           // its unknowns, 2 (hnx + 1)(hny + 1)
     const T* S[kMaxLv];
@@ -671,7 +671,6 @@ void BatchEngine<T>::build(cudaStream_t s) {
         b.pr = G.pr.template as<T>();
         b.pd = G.pd.template as<T>();
         b.r1 = G.r1.template as<T>();
-        b.e1 = G.e1.template as<T>();
         require(b.L >= 1 && b.L < kMaxLv, "batched solve: needs 1 to 11 h-coarsenings");
         for (int l = 0; l <= b.L; ++l) {
             HLevel<T>& H = G.h[l];
@@ -868,14 +867,17 @@ void BatchEngine<T>::build(cudaStream_t s) {
                 a.x_zero = k == 0 ? 1 : 0;
             }
         }
-        for (int r = 0; r < 4; ++r) {
-            upload(g.a[r], lo_a[r], s);
-            upload(g.a_hi[r], hi_a[r], s);
-            upload(g.f[r], fx[r], s);
+        for (int r = 0; r < 4; ++r) {   // the forms that capture_vcycle launches
+            if (sizeof(T) == 4 || !g.fix) upload(g.a[r], lo_a[r], s);
+            if (sizeof(T) == 4 && !g.fix) upload(g.a_hi[r], hi_a[r], s);
+            if (g.fix) upload(g.f[r], fx[r], s);
         }
-        upload(g.a_q, qa, s);
-        upload(g.f_q, fq, s);
-        upload(g.it_fix, fixed, s);
+        if (g.fix) {
+            upload(g.f_q, fq, s);
+            upload(g.it_fix, fixed, s);
+        } else {
+            upload(g.a_q, qa, s);
+        }
         g.n_fix = int(fixed.size());
         upload(g.it_lo, lo, s);
         upload(g.it_hi, hi, s);

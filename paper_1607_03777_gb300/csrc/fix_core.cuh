@@ -22,7 +22,7 @@
 // it enters the jumps of the lines m = 0 and the cross sums over them and nothing
 // else, and a translation of both sides of a face leaves nothing, whatever else moves
 // on top of it.  (With one exponent for all entries of an element, u_x = 1 and u_y of
-// size 1e-12 lost 38 of the 53 bits of what u_y gives, and a nearly rigid motion of a
+// size 1e-12 left 20 of the 53 bits of what u_y gives, and a nearly rigid motion of a
 // stiff inclusion is such a field; the separate exponents cost 2 to 10 % of an apply.)
 // Sums over one component are exact; a jump is formed on the coarser grid of the
 // face's two elements, the same on both sides.  Viscosities are 62-bit
@@ -267,9 +267,11 @@ FIX_HD i64 mulc(i64 x) {   // C x by shifts and additions
     else if constexpr (C == 1) return x;
     else if constexpr (C % 2 == 0) return mulc<C / 2>(x) << 1;
     else if constexpr (C == 3) return (x << 1) + x;
-    else return (x << 4) - x;   // 15
+    else {
+        static_assert(C == 15, "an odd factor without a form here (5, of A = 4: see tri)");
+        return (x << 4) - x;
+    }
 }
-static_assert(10 % 2 == 0, "10 = 2 * 5 is not covered by mulc: see tri()");
 template <int A>
 FIX_HD i64 tri(i64 x) {   // A (A + 1) / 2 x
     if constexpr (A == 4) return ((x << 2) + x) << 1;

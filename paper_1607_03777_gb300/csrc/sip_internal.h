@@ -153,6 +153,8 @@ Tab1D<N, T> make_tab() {
 enum ApplyVariant { APPLY_AUTO = 0, APPLY_ELEM2 = 1, APPLY_ELEM1 = 2, APPLY_TILE = 3, APPLY_STAGE = 4,
                     APPLY_WARP = 6, APPLY_FIX = 7 };
 
+constexpr int kSMs = 152;   // of a GB300
+
 struct OpGeom {
     int nx, ny;
     double hx, hy;

@@ -328,8 +328,9 @@ struct sip_problem {
     int k = 0, n = 0, nb = 0, mp = 0;
     int64_t ne = 0, n_u = 0, n_p = 0;
     sip::OpGeom geom{};      // the SIP operator of degree k
-    // Schedule of a Stokes solve whose viscosity contrast is above kFixedContrast:
-    // FP64 arithmetic in every operator.  There the saddle system's attainable
+    // Schedule of a Stokes solve whose viscosity contrast is above kFixedContrast, alone,
+    // grouped or served: FP64 arithmetic in every operator and in the FP32 cycle's marked
+    // tiles.  There the saddle system's attainable
     // residual in FP64 comes near the tolerances in use; a solve whose true residual
     // misses the tolerance when its recurrence meets it continues from rounding
     // errors, and the solution then depends on the operators' last bits: two equally

@@ -415,7 +415,7 @@ void bj_apply_n(int ne, const T* r, T* out, T* x, const int* emap, const T* cls_
     // 42.4 -> 33.9 us an apply); above k = 2 the FP64 pipe bounds both kernels and more
     // CTAs per SM win (k = 4: 141.6 against 146.8 us).
     if constexpr (sizeof(T) == 4 || N <= 3) {
-        const int resident = 152 * bj_ctas<N, T>();
+        const int resident = kSMs * bj_ctas<N, T>();
         if (blocks > 3 * resident) {
             launch_k(k_bj_stream<N, T>, unsigned(resident), 256, 0, s, a, blocks);
             SIP_CHECK_LAUNCH();
