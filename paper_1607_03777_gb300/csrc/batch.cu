@@ -590,13 +590,13 @@ struct BatchEngine {
     // groups run side by side within a stage: a stream per further one
     std::vector<cudaStream_t> side;
     std::vector<cudaEvent_t> ev;
-    // continuous levels in two launches each (hlevel.cu), where every level allows it
+    // continuous levels in two launches each (hlevel.cu), where that is the faster form
     struct Level {
+        bool fused = false;
         DeviceBuffer before, after, it_before, it_after;
         int n_before = 0, n_after = 0, t_before = 0, t_after = 0;
     };
     std::vector<Level> levels;
-    bool fused_levels = false;
     // work lists of the vector kernels
     DeviceBuffer it_u, it_parts, it_q1, it_v0, it_coarse;
     int n_u_items = 0, n_parts = 0, n_q1 = 0, n_v0 = 0, n_coarse = 0;
@@ -727,41 +727,42 @@ void BatchEngine<T>::build(cudaStream_t s) {
         n_lv[l] = int(a.size());
         n_lv1[l] = int(b1.size());
     }
-    fused_levels = true;
-    for (int m = 0; m < nmem; ++m)
-        for (int l = 0; l < hm[m].L; ++l)
-            fused_levels = fused_levels && fused_level_ok(mg(probs[m]).h[l], steps_h);
     levels.clear();
-    if (fused_levels) {
-        levels.resize(max_L);
-        for (int l = 0; l < max_L; ++l) {
-            std::vector<LevelArgs<T>> before(nmem), after(nmem);
-            std::vector<int2> ib, ia;
-            Level& V = levels[l];
-            int n = 0;
-            for (int m = 0; m < nmem; ++m) n += l < hm[m].L ? 1 : 0;
-            for (int m = 0; m < nmem; ++m) {
-                if (l >= hm[m].L) continue;
-                Multigrid<T>& G = mg(probs[m]);
-                HLevel<T>& H = G.h[l];
-                double c1[kMaxSt], c2[kMaxSt];
-                cheb_coefs(probs[m]->desc.cheb_lo * H.lmax, probs[m]->desc.cheb_hi * H.lmax, steps_h, c1, c2);
-                T* x0 = H.d.template as<T>();
-                before[m] = level_before_args<T>(H, G.h[l + 1], steps_h, c1, c2, x0, n);
-                after[m] = level_after_args<T>(H, G.h[l + 1], steps_h, c1, c2, x0, H.x.template as<T>(), n);
-                for (int t = 0; t < before[m].tiles; ++t) ib.push_back({m, t});
-                for (int t = 0; t < after[m].tiles; ++t) ia.push_back({m, t});
-                V.t_before = std::max(V.t_before, before[m].threads);
-                V.t_after = std::max(V.t_after, after[m].threads);
-            }
-            upload(V.before, before, s);
-            upload(V.after, after, s);
-            upload(V.it_before, ib, s);
-            upload(V.it_after, ia, s);
-            V.n_before = int(ib.size());
-            V.n_after = int(ia.size());
-            SIP_CUDA(cudaStreamSynchronize(s));   // staging vectors of this level
+    levels.resize(max_L);
+    for (int l = 0; l < max_L; ++l) {
+        std::vector<LevelArgs<T>> before(nmem), after(nmem);
+        std::vector<int2> ib, ia;
+        Level& V = levels[l];
+        int n = 0;
+        size_t vertices = 0;
+        for (int m = 0; m < nmem; ++m) {
+            if (l >= hm[m].L) continue;
+            ++n;
+            vertices += size_t(hm[m].hn[l]) / 2;
         }
+        V.fused = fused_level_ok<T>(steps_h, vertices);
+        if (!V.fused) continue;
+        for (int m = 0; m < nmem; ++m) {
+            if (l >= hm[m].L) continue;
+            Multigrid<T>& G = mg(probs[m]);
+            HLevel<T>& H = G.h[l];
+            double c1[kMaxSt], c2[kMaxSt];
+            cheb_coefs(probs[m]->desc.cheb_lo * H.lmax, probs[m]->desc.cheb_hi * H.lmax, steps_h, c1, c2);
+            T* x0 = H.d.template as<T>();
+            before[m] = level_before_args<T>(H, G.h[l + 1], steps_h, c1, c2, x0, n);
+            after[m] = level_after_args<T>(H, G.h[l + 1], steps_h, c1, c2, x0, H.x.template as<T>(), n);
+            for (int t = 0; t < before[m].tiles; ++t) ib.push_back({m, t});
+            for (int t = 0; t < after[m].tiles; ++t) ia.push_back({m, t});
+            V.t_before = std::max(V.t_before, before[m].threads);
+            V.t_after = std::max(V.t_after, after[m].threads);
+        }
+        upload(V.before, before, s);
+        upload(V.after, after, s);
+        upload(V.it_before, ib, s);
+        upload(V.it_after, ia, s);
+        V.n_before = int(ib.size());
+        V.n_after = int(ia.size());
+        SIP_CUDA(cudaStreamSynchronize(s));   // staging vectors of this level
     }
     upload(d_mem, hm, s);
     upload(it_u, items_u, s);
@@ -962,7 +963,7 @@ void BatchEngine<T>::capture_vcycle(cudaStream_t s) {
     launch_k(k_b_rdc<T>, dim3(unsigned(n_v0)), kChunk, 0, s, mb, it_v0.template as<int2>(), act);
     SIP_CHECK_LAUNCH();
     for (int l = 0; l < max_L; ++l) {   // members with l < L go one level down
-        if (fused_levels) {
+        if (levels[l].fused) {
             Level& V = levels[l];
             launch_level_batch<T>(false, V.before.template as<LevelArgs<T>>(), V.it_before.template as<int2>(),
                                   V.n_before, V.t_before, act, s);
@@ -979,7 +980,7 @@ void BatchEngine<T>::capture_vcycle(cudaStream_t s) {
     launch_k(k_b_coarse<T>, dim3(unsigned(n_coarse)), kChunk, 0, s, mb, it_coarse.template as<int2>(), act);
     SIP_CHECK_LAUNCH();
     for (int l = max_L - 1; l >= 0; --l) {
-        if (fused_levels) {
+        if (levels[l].fused) {
             Level& V = levels[l];
             launch_level_batch<T>(true, V.after.template as<LevelArgs<T>>(), V.it_after.template as<int2>(),
                                   V.n_after, V.t_after, act, s);

@@ -8,9 +8,9 @@
 // a halo that shrinks by one ring per application, one thread per (vertex,
 // component) with its stencil row in registers (read once instead of once per
 // step) and the direction in shared memory.  The rings are recomputed by the
-// neighbouring tiles: 2.0x the FP64 work at 12 x 12 vertices and three steps,
-// which is what limits the tile from below; large FP64 levels, where that work
-// outweighs the launches, keep one launch per step (fused_level_ok).
+// neighbouring tiles: 2.0x the stencil work at 12 x 12 vertices and three steps,
+// which is what limits the tile from below; FP64 levels where that work
+// outweighs the launches keep one launch per step (fused_level_ok).
 #include "sip_internal.h"
 #include "sip_level.cuh"
 #include "sip_solver.h"
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kMaxThreads) k_level_batch(const LevelArgs<T>*
 }
 
 // Coarse vertices per tile and direction: the largest (least recomputation)
-// that still gives most SMs a tile.
+// that still gives most SMs (110 of 152) a tile.
 int level_tile(int nvxc, int nvyc, int steps, int members) {
     for (int t = 6; t > 2; --t) {
         const int rw = 2 * t + 1 + 2 * steps;
@@ -214,10 +214,15 @@ inline int round32(int n) { return (n + 31) / 32 * 32; }
 
 }  // namespace
 
+// FP64: the recomputed rings cost more than the launches they save from about 130^2
+// vertices on, over all members of a batch.  V-cycle, k = 1, two launches per level / one
+// per step: 128^2 elements 164 / 179 us, 144^2 222 / 211, 192^2 268 / 232, 256^2 429 / 384;
+// grouped batches, k = 2: 4 x 64^2 48.1 / 50.7 ms, 16 x 32^2 62.9 / 61.8, 8 x 64^2 86.7 / 83.3,
+// 8 x 128^2 259 / 239.  FP32: 256^2 126 / 152 us, 512^2 352 / 351.
 template <typename T>
-bool fused_level_ok(const HLevel<T>& L, int steps) {
+bool fused_level_ok(int steps, size_t vertices) {
     if (steps < 1 || steps > kLevelSteps) return false;
-    return sizeof(T) == 4 || size_t(L.nvx) * L.nvy <= size_t(300) * 300;
+    return sizeof(T) == 4 || vertices <= 17000;
 }
 
 template <typename T>
@@ -267,7 +272,7 @@ void launch_level_batch(bool after, const LevelArgs<T>* args, const int2* items,
 }
 
 #define SIP_LEVEL(T)                                                                              \
-    template bool fused_level_ok<T>(const HLevel<T>&, int);                                       \
+    template bool fused_level_ok<T>(int, size_t);                                                 \
     template LevelArgs<T> level_before_args<T>(HLevel<T>&, HLevel<T>&, int, const double*,        \
                                                const double*, T*, int);                           \
     template LevelArgs<T> level_after_args<T>(HLevel<T>&, HLevel<T>&, int, const double*,         \

@@ -132,7 +132,8 @@ struct HLevel {
 
 // ---- hlevel.cu: a level's work before and after its coarse correction, one
 // launch each (Chebyshev coefficients c1, c2 per step; x, xin: iterate buffers
-// that differ).  fused_level_ok: number of steps and level size it serves.
+// that differ).  fused_level_ok: the numbers of steps, and of vertices over all levels
+// that share the launch, where it is the faster form.
 constexpr int kLevelSteps = 4;
 template <typename T>
 struct LevelArgs {
@@ -149,7 +150,7 @@ struct LevelArgs {
     int steps, tile, rw;   // coarse vertices of a tile, vertices of its region, per direction
     int tiles, threads;    // CTAs and threads per CTA
 };
-template <typename T> bool fused_level_ok(const HLevel<T>& L, int steps);
+template <typename T> bool fused_level_ok(int steps, size_t vertices);
 // members: number of levels that share the launch (more members, larger tiles)
 template <typename T>
 LevelArgs<T> level_before_args(HLevel<T>& L, HLevel<T>& C, int steps, const double* c1, const double* c2,

@@ -819,7 +819,7 @@ void Multigrid<T>::hcycle(int l, cudaStream_t s) {
     }
     HLevel<T>& C = h[l + 1];
     const int steps = P->desc.cheb_steps_h;
-    if (fused_level_ok(Lv, steps)) {
+    if (fused_level_ok<T>(steps, size_t(Lv.nvx) * Lv.nvy)) {
         const Cheb ch(P->desc.cheb_lo * Lv.lmax, P->desc.cheb_hi * Lv.lmax);
         double c1[kLevelSteps], c2[kLevelSteps];
         c1[0] = 0.0;
