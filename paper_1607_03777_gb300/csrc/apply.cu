@@ -500,7 +500,7 @@ void launch_apply_sip(int N, const OpGeom& g, const T* x, T* y, const T* eta, T 
     }
     bool fix = false;
     if constexpr (sizeof(T) == 8) {
-        fix = fixed_point(g, v);
+        fix = fixed_point(N, g, v);
         if (fix && launch_apply_fix(N, g, x, y, eta, alpha, z, beta, nullptr, s)) return;
     }
     // factors outside the fixed-point range (meshes of extreme aspect): the staged kernel

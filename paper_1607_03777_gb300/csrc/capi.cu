@@ -229,7 +229,7 @@ sip_status sip_problem_schedule(const sip_problem* p, int apply[2], int fused[2]
     for (int t = 0; t < 2; ++t) {
         if (apply) {
             const int v = p->geom.variant[t];
-            if (t == 0 && p->n <= 6 && sip::fixed_point(p->geom, v)) apply[t] = 4;
+            if (t == 0 && p->n <= 6 && sip::fixed_point(p->n, p->geom, v)) apply[t] = 4;
             else if (v == sip::APPLY_STAGE) apply[t] = t == 0 || p->geom.stage_rows[t] == 4 ? 5 : 4;
             else apply[t] = v != sip::APPLY_AUTO ? v : int(p->n <= 6 ? sip::APPLY_ELEM2 : sip::APPLY_TILE);
             if (t == 1 && p->geom.n_hi > 0 && p->n <= 6) apply[t] = int(sip::APPLY_STAGE);

@@ -160,8 +160,8 @@ struct OpGeom {
     double hx, hy;
     int bc[4];
     double pen_x, pen_y;
-    // ApplyVariant (APPLY_AUTO: FP64 fixed point unless fp64 is set, else component-split,
-    // for N <= 6; above the tile kernel)
+    // ApplyVariant (APPLY_AUTO: FP64 see fixed_point, else component-split, for N <= 6;
+    // above the tile kernel)
     int variant[2];
     int fused[2];     // p-level smoother step fused into one launch (1) or not (0)
     int stage_rows[2];   // tile rows of the staged apply (2 or 4), per precision
@@ -202,8 +202,13 @@ inline void set_apply_code(OpGeom& g, int t, int code) {
     g.stage_rows[t] = code == 5 ? 4 : 2;
     if (t == 0) g.fp64 = code != 4;
 }
-// The FP64 operator runs in fixed point under variant v.
-inline bool fixed_point(const OpGeom& g, int v) { return v == APPLY_FIX || (v == APPLY_AUTO && !g.fp64); }
+// The FP64 operator of degree N - 1 runs in fixed point under variant v.  Its default is
+// the component-split kernel where that is faster, at degree 1 on small meshes (32^2 10.4
+// us, fixed point 11.4; 96^2 10.1 / 12.2, 128^2 16.2 / 12.8; degree 2, 32^2 15.6 / 14.5).
+inline bool fixed_point(int N, const OpGeom& g, int v) {
+    if (v == APPLY_AUTO) return !g.fp64 && (N > 2 || (long long)g.nx * g.ny > 12000);
+    return v == APPLY_FIX;
+}
 
 // y = alpha * (A x) + beta * z (z may be null).  N = polynomial degree + 1
 // of the space the operator acts on (N = 2 for the Galerkin A_1).

@@ -494,7 +494,7 @@ bool Multigrid<T>::residual_restrict(const T* y, const T* b, T* r1, cudaStream_t
     const int v = apply_variant<T>(P->op());
     bool fix = false;
     if constexpr (sizeof(T) == 8) {
-        fix = fixed_point(P->op(), v);
+        fix = fixed_point(N, P->op(), v);
         if (fix && launch_apply_fix(N, P->op(), y, nullptr, eta_of<T>(P), -1.0, b, 1.0, r1, s)) return true;
     }
     if (split || fix || v == APPLY_STAGE)
@@ -532,7 +532,7 @@ void Multigrid<T>::setup(cudaStream_t s) {
 
     const OpGeom& g1 = P->geom1;
     OpGeom g0 = P->geom;   // probing for A_0: FP64 arithmetic, as for A_1
-    if (fixed_point(g0, g0.variant[0])) g0.variant[0] = APPLY_ELEM2;
+    if (fixed_point(N, g0, g0.variant[0])) g0.variant[0] = APPLY_ELEM2;
     const bool q0 = d.coarse == SIP_COARSE_Q0;
     if (d.n_hlevels == 0 && !q0) {
         // A_p(Q^2_1): the coarse problem A_1 = P^T A P itself, by probing with
@@ -1125,7 +1125,7 @@ sip_status run_solve(sip_problem* P, const double* f_u, const double* g_p, doubl
     // y = K v  (w_u = A v_u + B v_p, w_p = B^T v_u), one application per outer
     // iteration: FP64 arithmetic at every contrast
     OpGeom gK = P->op();
-    if (fixed_point(gK, gK.variant[0])) gK.variant[0] = APPLY_ELEM2;
+    if (fixed_point(P->n, gK, gK.variant[0])) gK.variant[0] = APPLY_ELEM2;
     auto applyK = [&](const double* v, double* y) {
         launch_apply_B<double>(P->k, P->op(), v + n_u, W.tu.as<double>(), s);
         launch_apply_sip<double>(P->n, gK, v, y, eta, 1.0, W.tu.as<double>(), 1.0, s);

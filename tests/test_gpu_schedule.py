@@ -78,3 +78,17 @@ def test_unpinned_runs_the_default_again(ctx):
         q.apply_B(p, out)
     assert a.schedule() == b.schedule()
     assert torch.equal(y[1], y[2]) and not torch.equal(y[0], y[1])
+
+
+@pytest.mark.parametrize("k,n,code", [(1, 32, 1), (1, 109, 1), (1, 110, 4), (1, 128, 4), (2, 8, 4), (5, 3, 4)])
+def test_default_before_setup(ctx, k, n, code):
+    """A problem that was not set up reports and runs the default: fixed point, but at degree
+    1 on small meshes the component-split kernel."""
+    prob = api.Problem(ctx, n, n, k, synth.random_eta(n * n, 3, (0.0, 3.0)), bc=synth.SINKER_BC)
+    u = torch.from_numpy(synth.random_vector(prob.n_u, 4)).cuda()
+    y = [torch.empty_like(u) for _ in range(2)]
+    prob.apply_A(u, y[0])
+    assert prob.schedule()["apply"][0] == code
+    prob.set_schedule(apply=[code, 0])
+    prob.apply_A(u, y[1])
+    assert torch.equal(*y)
