@@ -5,7 +5,8 @@
 // normal and multiplies the zeros of the 1D tables; one thread per (element,
 // line) forms a line's scaled entries, their even and odd sums (both end
 // traces) and their prefix sums (int l_p l_q' = 2 l_p(1) l_q(1) for q > p, q - p
-// odd) once: about 35 FP64 operations per line at k = 4 instead of 230.
+// odd) once: 37 (B) and 41 (B^T) FP64 operations per line at k = 4 instead of 230, and
+// the FP64 pipe 84 and 80 % busy (512^2).
 // 250 x 190, k = 4, both operators: 417 us before, 72 now.
 //
 // Mode q receives (h / 2) l_q(1) (f_1 - (-1)^q f_0 - 2 sum of the other parity beyond q) with

@@ -3,17 +3,24 @@
 // sip_solver.h), and the part of the FP32 operator that needs
 // FP64 arithmetic (split precision: FP32 storage, the tiles of hi_tiles).
 //
-// What bounds it: the integer pipes (about 4000 wide multiply-adds and
-// 64-bit additions per element at k = 3); FP64 only converts (one multiply and
-// one conversion per entry in and out, 128 operations per element against the
-// 933 of the FP64 kernel, on a pipe that does 2 per SM and clock).
+// What bounds it: instruction fetch and the latency of integer chains with the 12 to
+// 16 warps per SM that shared memory admits (first stalls no_instruction and wait; the
+// ALU pipe 50 % busy, the FP64 pipe 35 %, 47 % of the issue slots used at 512^2, k = 4).
+// 17.6 thousand integer thread instructions per element at k = 3, 25.8 at k = 4.
+// FP64 only converts, one multiply and one conversion per entry in (the halo's too:
+// 1.5 times the tile's entries at 8 x 8, 1.75 at 8 x 4) and out: 173 operations per
+// element at k = 3, 291 at k = 4, against the 933 of the FP64 kernel at k = 3, on a pipe
+// that does 2 per SM and clock.  128^2, k = 3: 20.8 us, FP64 kernels 41.6; 512^2, k = 4:
+// 467 and 736 us.
 //
 // Layout: a CTA serves a tile of TW x TH elements with one thread per
 // (element, line), both components; a warp shares its line index, lanes are
 // elements.  The tile's and halo's entries are read once, a warp per element
 // with consecutive lanes on consecutive entries, converted and kept in shared
-// memory as integers; traces of all faces go beside them, then rows and
-// columns are two passes, and the results leave as consecutive stores.
+// memory as integers; traces of all faces and the constant modes' jumps, once per
+// face, go beside them, then rows and columns are two passes, and the results leave
+// as consecutive stores.  (Jumps formed by each line that uses them cost 9 to 20 % more
+// than once per face, and per element a CTA per SM at k = 4.)
 #include "fix_core.cuh"
 #include "sip_elem.cuh"
 #include "sip_face.cuh"

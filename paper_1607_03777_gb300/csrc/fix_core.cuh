@@ -1,9 +1,9 @@
 // FP64-accurate SIP apply in 64-bit fixed point (eq. stiffness_form).
 //
 // Why: GB300 executes 2 FP64 operations per SM and clock, but 64 integer
-// additions and about 11 wide integer multiply-adds (measured: DFMA, DADD,
-// DMUL, FP64 <-> integer conversions 1.6-1.9 lanes per clock and SM, a 64-bit
-// addition 46, mad.wide.s32 11).  In the unnormalised Legendre basis the 1D
+// additions and 12 wide integer multiply-adds (measured lanes per clock and SM: DFMA and
+// FP64 <-> integer conversions 2.0, DADD and DMUL 1.7, a 64-bit addition about 45,
+// mad.wide.s32 12).  In the unnormalised Legendre basis the 1D
 // factors of the operator are small integers: P_i(+-1) = (+-1)^i,
 // P_i'(+-1) = (+-1)^(i+1) i(i+1)/2, int P_a' P_b' = m(m+1), int P_p P_q' = 2,
 // so traces, jumps, strains and the lifting of the face terms need additions
