@@ -10,8 +10,8 @@
 // FP64 only converts, one multiply and one conversion per entry in (the halo's too:
 // 1.5 times the tile's entries at 8 x 8, 1.75 at 8 x 4) and out: 173 operations per
 // element at k = 3, 291 at k = 4, against the 933 of the FP64 kernel at k = 3, on a pipe
-// that does 2 per SM and clock.  128^2, k = 3: 20.8 us, FP64 kernels 41.6; 512^2, k = 4:
-// 467 and 736 us.
+// that does 2 per SM and clock.  128^2, k = 3: 20.5 us, FP64 kernels 41.6; 512^2, k = 4:
+// 459 and 736 us; 64^2, k = 3: 13.6 us.
 //
 // Layout: a CTA serves a tile of TW x TH elements with one thread per
 // (element, line), both components; a warp shares its line index, lanes are

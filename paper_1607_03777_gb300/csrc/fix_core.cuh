@@ -457,8 +457,12 @@ FIX_HD void phase_traces(int tid, const Mesh& g, i64* sm) {
         }
         se[L::I_R + el] = expo_pack(E, E + R);
     }
-    for (int f = tid; f < L::NF; f += L::NT)
-        mean_jumps<N, TW, TH>(g, su, se, f, sm + L::O_M, reinterpret_cast<short*>(se + L::I_M));
+    // from the last thread down: the first ones have the halo's traces below
+#pragma unroll
+    for (int r = 0; r < (L::NF + L::NT - 1) / L::NT; ++r) {
+        const int f = r * L::NT + L::NT - 1 - tid;
+        if (f < L::NF) mean_jumps<N, TW, TH>(g, su, se, f, sm + L::O_M, reinterpret_cast<short*>(se + L::I_M));
+    }
 #pragma unroll
     for (int dir = 0; dir < 2; ++dir)
 #pragma unroll
