@@ -2,14 +2,14 @@
 // the coarse correction (Chebyshev / point-Jacobi steps from zero, residual,
 // restriction) and everything after it (interpolation, steps).
 //
-// What bounds it: latency.  A stencil application on a 129^2-vertex level is
+// What bounds it: launches and latency.  A stencil application on a 129^2-vertex level is
 // 1 us of FP64 work and 4 MB from L2, but one launch per step takes about 4 us
 // in a replayed graph, nine per level.  Here a CTA runs all steps of its tile on
 // a halo that shrinks by one ring per application, one thread per (vertex,
 // component) with its stencil row in registers (read once instead of once per
 // step) and the direction in shared memory.  The rings are recomputed by the
-// neighbouring tiles: 2.0x the stencil work at 12 x 12 vertices and three steps,
-// which is what limits the tile from below; FP64 levels where that work
+// neighbouring tiles: with three steps 1.6 (before) and 1.4 (after) stencil rows per row
+// kept at 12 x 12 vertices, 3.2 and 2.4 at 4 x 4; FP64 levels where that work
 // outweighs the launches keep one launch per step (fused_level_ok).  On 129^2 vertices
 // the FP64 pipe is 76 % busy.
 #include "sip_internal.h"
