@@ -98,3 +98,26 @@ def test_marked_tiles_of_the_fp32_cycle(ctx, k, inner_loop):
     Q.setup()
     Q.apply_A_f32(x, y[2])
     assert torch.equal(y[0], y[2])
+
+
+@pytest.mark.parametrize("contrast", [1e2, 1e3])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_fixed_point_and_fp64_do_not_mix(ctx, contrast, precision):
+    """With the fixed-point kernel pinned a stiff problem's viscous solves run it and its
+    Stokes solves FP64 kernels: neither leaves its schedule behind for the other."""
+    def fresh():
+        P, f = problem(ctx, 32, 2, contrast, precision, code=4)
+        P.set_schedule(fused=[0, 0])   # bits do not depend on the autotuner
+        return P, f
+
+    def viscous(P, f):
+        x = torch.as_tensor(synth.random_vector(P.n_u, 5)).cuda()
+        y = torch.empty_like(x)
+        P.inner_solve(x, y, rtol=1e-3)
+        return y
+
+    s0, v0 = solve(*fresh()), viscous(*fresh())
+    P, Q = fresh(), fresh()
+    for _ in range(2):
+        assert torch.equal(solve(*P), s0) and torch.equal(viscous(*Q), v0)
+        assert torch.equal(viscous(*P), v0) and torch.equal(solve(*Q), s0)
