@@ -8,8 +8,8 @@
 // ALU pipe 50 % busy, the FP64 pipe 35 %, 47 % of the issue slots used at 512^2, k = 4).
 // 17.6 thousand integer thread instructions per element at k = 3, 25.8 at k = 4.
 // FP64 only converts, one multiply and one conversion per entry in (the halo's too:
-// 1.5 times the tile's entries at 8 x 8, 1.75 at 8 x 4) and out: 173 operations per
-// element at k = 3, 291 at k = 4, against the 933 of the FP64 kernel at k = 3, on a pipe
+// 1.5 times the tile's entries at 8 x 8, 1.75 at 8 x 4) and out: 171 operations per
+// element at k = 3, 289 at k = 4, against the 933 of the FP64 kernel at k = 3, on a pipe
 // that does 2 per SM and clock.  128^2, k = 3: 20.5 us, FP64 kernels 41.6; 512^2, k = 4:
 // 459 and 736 us; 64^2, k = 3: 13.6 us.
 //
